@@ -590,7 +590,8 @@ int svt_server_bench_poisson(svt_server server, const uint32_t *h_pool, const ui
  * with hand-written forward and backward kernels, for calibrating fit
  * constants on tracks whose true parameters theta are known.  Tracks are
  * used in sector order: svt_calib_index sorts them (stable counting sort on
- * the device) and svt_calib_gather permutes per-track arrays.  All sums run
+ * the device), svt_calib_sort puts the tracks in that order as well and
+ * svt_calib_gather permutes per-track arrays.  All sums run
  * in a fixed order, so repeated calls give identical bits.
  * Layouts: x float [N][6], theta float [N][3], w float [3], y float [N][6].
  * ====================================================================== */
@@ -604,6 +605,15 @@ size_t svt_calib_index_size(uint64_t n_tracks, uint32_t n_sectors);
  * n_sectors <= 512. */
 int svt_calib_index(const int32_t *d_sector, uint64_t n_tracks, uint32_t n_sectors, void *d_index,
                     size_t index_bytes, int32_t *d_perm, uint64_t *d_status, void *stream);
+
+/* svt_calib_index together with the tracks themselves in sector order, in the
+ * same pass: d_out_x[i] = d_x[d_perm[i]] (6 floats), d_out_theta[i] =
+ * d_theta[d_perm[i]] (3 floats).  d_out_x must be 8-byte aligned; no output may
+ * overlap an input.  Tracks of a bad sector (see d_status) are left out. */
+int svt_calib_sort(const float *d_x, const float *d_theta, const int32_t *d_sector,
+                   uint64_t n_tracks, uint32_t n_sectors, void *d_index, size_t index_bytes,
+                   int32_t *d_perm, float *d_out_x, float *d_out_theta, uint64_t *d_status,
+                   void *stream);
 
 /* d_dst[i][c] = d_src[d_perm[i]][c] for c < width. */
 int svt_calib_gather(const float *d_src, uint32_t width, const int32_t *d_perm, uint64_t n,

@@ -135,6 +135,8 @@ SIGNATURES = {
                                                 _vp, _vp, _vp, ctypes.POINTER(ctypes.c_double)]),
     "svt_calib_index_size": (_sz, [_u64, _u32]),
     "svt_calib_index": (ctypes.c_int, [_vp, _u64, _u32, _vp, _sz, _vp, _vp, _vp]),
+    "svt_calib_sort": (ctypes.c_int, [_vp, _vp, _vp, _u64, _u32, _vp, _sz, _vp, _vp, _vp, _vp,
+                                      _vp]),
     "svt_calib_gather": (ctypes.c_int, [_vp, _u32, _vp, _u64, _vp, _vp]),
     "svt_calib_workspace_size": (_sz, [_u64, _u32]),
     "svt_calib_forward": (ctypes.c_int, [_vp, _u64, _u32, _vp, _vp, _vp, _vp, _vp]),

@@ -37,18 +37,14 @@ class CalibData:
                                  device=device)
         self.perm = torch.empty(max(n, 1), dtype=torch.int32, device=device)
         status = torch.empty(1, dtype=torch.int64, device=device)
-        st = _stream(None)
-        N.check(L.svt_calib_index(_p(sector), n, self.n_sectors, _p(self.index),
-                                  self.index.numel(), _p(self.perm), _p(status), st),
-                "svt_calib_index")
+        self.x = torch.empty((max(n, 1), 6), dtype=torch.float32, device=device)
+        self.theta = torch.empty((max(n, 1), 3), dtype=torch.float32, device=device)
+        N.check(L.svt_calib_sort(_p(x), _p(theta), _p(sector), n, self.n_sectors, _p(self.index),
+                                 self.index.numel(), _p(self.perm), _p(self.x), _p(self.theta),
+                                 _p(status), _stream(None)), "svt_calib_sort")
         key = int(status.cpu().numpy().view(np.uint64)[0])
         if key != N.STATUS_OK:
             raise N.SvtError(f"bad sector at track {key >> 8}")
-        self.x = torch.empty((max(n, 1), 6), dtype=torch.float32, device=device)
-        self.theta = torch.empty((max(n, 1), 3), dtype=torch.float32, device=device)
-        N.check(L.svt_calib_gather(_p(x), 6, _p(self.perm), n, _p(self.x), st), "svt_calib_gather")
-        N.check(L.svt_calib_gather(_p(theta), 3, _p(self.perm), n, _p(self.theta), st),
-                "svt_calib_gather")
         self.w = (torch.ones(3) if w is None else torch.as_tensor(w)).to(device, torch.float32).contiguous()
         # zero-filled once: the fused pass keeps its tickets here
         self.workspace = torch.zeros(L.svt_calib_workspace_size(n, self.n_sectors), dtype=torch.uint8,

@@ -136,7 +136,7 @@ RunWs carve_run(void *base, uint64_t max_words, uint64_t max_events, uint64_t ro
 
 // Sector index of the calibration tracks.
 struct CalibIndex {
-    uint32_t *counts;
+    uint32_t *counts, *totals;
     int32_t *sector_off, *sector_item, *item_sector, *item_start, *n_items;
     uint32_t max_items;
     size_t bytes;
@@ -146,6 +146,7 @@ CalibIndex carve_calib_index(const void *base, uint64_t n, uint32_t S) {
     CalibIndex x;
     x.max_items = calib_max_items(n, S);
     x.counts = c.take<uint32_t>((size_t)S * calib_tiles(n) + 1);
+    x.totals = c.take<uint32_t>(S);
     x.sector_off = c.take<int32_t>(S + 1);
     x.sector_item = c.take<int32_t>(S + 1);
     x.item_sector = c.take<int32_t>(x.max_items);
@@ -705,24 +706,53 @@ size_t svt_calib_index_size(uint64_t n_tracks, uint32_t n_sectors) {
     return carve_calib_index(nullptr, n_tracks, n_sectors).bytes;
 }
 
-int svt_calib_index(const int32_t *d_sector, uint64_t n_tracks, uint32_t n_sectors, void *d_index,
-                    size_t index_bytes, int32_t *d_perm, uint64_t *d_status, void *stream) {
+}  // extern "C"
+
+namespace {
+
+int calib_sort(const float *d_x, const float *d_theta, const int32_t *d_sector, uint64_t n_tracks,
+               uint32_t n_sectors, void *d_index, size_t index_bytes, int32_t *d_perm,
+               float *d_out_x, float *d_out_theta, uint64_t *d_status, cudaStream_t st) {
     if (!calib_sizes_ok(n_tracks, n_sectors) || !d_index || !d_status) return SVT_ERR_BAD_ARG;
     if (n_tracks > 0 && (!d_sector || !d_perm)) return SVT_ERR_BAD_ARG;
     CalibIndex x = carve_calib_index(d_index, n_tracks, n_sectors);
     if (index_bytes < x.bytes) return SVT_ERR_BAD_ARG;
-    cudaStream_t st = (cudaStream_t)stream;
-    unsigned long long *status = (unsigned long long *)d_status;
-    launch_prologue(nullptr, 0, 0, nullptr, nullptr, nullptr, status, nullptr, 0, nullptr, 0,
-                    nullptr, nullptr, 1, st);
-    if (cudaMemsetAsync(x.sector_off, 0, sizeof(int32_t) * (n_sectors + 1), st) != cudaSuccess ||
-        cudaMemsetAsync(x.sector_item, 0, sizeof(int32_t) * (n_sectors + 1), st) != cudaSuccess ||
-        cudaMemsetAsync(x.n_items, 0, sizeof(int32_t), st) != cudaSuccess)
-        return SVT_ERR_CUDA;
-    launch_calib_sort(d_sector, n_tracks, n_sectors, x.counts, d_perm, x.sector_off,
-                      x.sector_item, x.item_sector, x.item_start, x.n_items, status, tile_grid(),
-                      st);
-    return launch_status();
+    if (cudaMemsetAsync(d_status, 0xFF, sizeof(uint64_t), st) != cudaSuccess) return SVT_ERR_CUDA;
+    if (n_tracks == 0)
+        return cudaMemsetAsync(x.sector_off, 0, sizeof(int32_t) * (n_sectors + 1), st) ==
+                           cudaSuccess &&
+                       cudaMemsetAsync(x.sector_item, 0, sizeof(int32_t) * (n_sectors + 1), st) ==
+                           cudaSuccess &&
+                       cudaMemsetAsync(x.n_items, 0, sizeof(int32_t), st) == cudaSuccess
+                   ? SVT_OK
+                   : SVT_ERR_CUDA;
+    return launch_calib_sort(d_sector, n_tracks, n_sectors, x.counts, x.totals, d_perm,
+                             x.sector_off, x.sector_item, x.item_sector, x.item_start, x.n_items,
+                             d_x, d_theta, d_out_x, d_out_theta, (unsigned long long *)d_status,
+                             current_sm_count(), st) == cudaSuccess
+               ? SVT_OK
+               : SVT_ERR_CUDA;
+}
+
+}  // namespace
+
+extern "C" {
+
+int svt_calib_index(const int32_t *d_sector, uint64_t n_tracks, uint32_t n_sectors, void *d_index,
+                    size_t index_bytes, int32_t *d_perm, uint64_t *d_status, void *stream) {
+    return calib_sort(nullptr, nullptr, d_sector, n_tracks, n_sectors, d_index, index_bytes, d_perm,
+                      nullptr, nullptr, d_status, (cudaStream_t)stream);
+}
+
+int svt_calib_sort(const float *d_x, const float *d_theta, const int32_t *d_sector,
+                   uint64_t n_tracks, uint32_t n_sectors, void *d_index, size_t index_bytes,
+                   int32_t *d_perm, float *d_out_x, float *d_out_theta, uint64_t *d_status,
+                   void *stream) {
+    if (n_tracks > 0 &&
+        (!d_x || !d_theta || !d_out_x || !d_out_theta || ((uintptr_t)d_out_x & 7u)))
+        return SVT_ERR_BAD_ARG;
+    return calib_sort(d_x, d_theta, d_sector, n_tracks, n_sectors, d_index, index_bytes, d_perm,
+                      d_out_x, d_out_theta, d_status, (cudaStream_t)stream);
 }
 
 int svt_calib_gather(const float *d_src, uint32_t width, const int32_t *d_perm, uint64_t n,

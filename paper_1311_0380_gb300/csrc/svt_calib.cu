@@ -5,7 +5,7 @@
 //     L   = (1/N) sum_t [ sum_{k<3} w_k (y_tk - theta_tk)^2 + sum_{k>=3} y_tk^2 ]
 // with hand-written forward and backward kernels.
 //
-// Tracks are first sorted by sector (stable counting sort on the device);
+// Tracks are first put in sector order (stable counting sort on the device);
 // every kernel then works on "items" of at most CALIB_CHUNK consecutive tracks
 // of one sector: the forward, the loss alone and the general backward take
 // one warp per item, the fused loss-and-gradient pass a contiguous run of
@@ -22,7 +22,7 @@ namespace svt {
 namespace {
 
 constexpr int CALIB_CHUNK = 256;          // tracks per item (8 per lane)
-constexpr int SORT_TILE = 1024;           // tracks per histogram tile
+constexpr int SORT_TILE = 2048;           // tracks per tile of the sort
 constexpr int NPAR = 42;                  // 36 entries of F[s] + 6 of q[s]
 
 
@@ -33,116 +33,233 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 // ---- stable counting sort by sector ------------------------------------------
-__global__ void k_hist(const int32_t *__restrict__ sector, uint64_t n, uint32_t S, uint32_t T,
-                       uint32_t *counts, unsigned long long *status) {
+// Four passes: histograms of tiles of SORT_TILE tracks, a scan of every
+// sector's counts over the tiles (a block per sector), the sector offsets and
+// the item table, and the scatter.  The scans of all sectors in one block had
+// been 954 of the 1112 us of putting 4 M tracks in order; now the sort is
+// bound by moving the tracks (see k_scatter).
+constexpr int SORT_THREADS = 256, SORT_WARPS = SORT_THREADS / 32;
+constexpr int SORT_ROUNDS = SORT_TILE / SORT_THREADS;   // tracks per thread
+
+__global__ void __launch_bounds__(SORT_THREADS)
+    k_hist(const int32_t *__restrict__ sector, uint64_t n, uint32_t S, uint32_t T,
+           uint32_t *counts, unsigned long long *status) {
     __shared__ uint32_t h[512];
+    allow_next_grid();
     for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
-        for (uint32_t s = threadIdx.x; s < S; s += blockDim.x) h[s] = 0;
-        __syncthreads();
-        for (uint32_t j = threadIdx.x; j < SORT_TILE; j += blockDim.x) {
-            const uint64_t i = (uint64_t)t * SORT_TILE + j;
-            if (i < n) {
-                const int32_t s = sector[i];
-                if (s < 0 || (uint32_t)s >= S) {
-                    report(status, i, SVT_ERR_BAD_SECTOR);
-                } else {
-                    atomicAdd(&h[s], 1u);
-                }
-            }
+        for (uint32_t s = threadIdx.x; s < S; s += SORT_THREADS) h[s] = 0;
+        int32_t key[SORT_ROUNDS];   // every load of the tile in flight at once
+#pragma unroll
+        for (int r = 0; r < SORT_ROUNDS; ++r) {
+            const uint64_t i = (uint64_t)t * SORT_TILE + r * SORT_THREADS + threadIdx.x;
+            key[r] = i < n ? __ldg(sector + i) : 0;
         }
         __syncthreads();
-        for (uint32_t s = threadIdx.x; s < S; s += blockDim.x) counts[(uint64_t)s * T + t] = h[s];
+#pragma unroll
+        for (int r = 0; r < SORT_ROUNDS; ++r) {
+            const uint64_t i = (uint64_t)t * SORT_TILE + r * SORT_THREADS + threadIdx.x;
+            if (i >= n) continue;
+            if ((uint32_t)key[r] >= S)
+                report(status, i, SVT_ERR_BAD_SECTOR);
+            else
+                atomicAdd(&h[key[r]], 1u);
+        }
+        __syncthreads();
+        for (uint32_t s = threadIdx.x; s < S; s += SORT_THREADS) counts[(uint64_t)s * T + t] = h[s];
         __syncthreads();
     }
 }
 
-// exclusive scan of counts[0..n) in one block; n = S * T
-__global__ void __launch_bounds__(1024) k_scan_counts(uint32_t *counts, uint64_t n) {
-    __shared__ uint32_t sm[33];
+// block s: exclusive scan of sector s's counts over the tiles, and its total
+__global__ void __launch_bounds__(SORT_THREADS)
+    k_sector_scan(uint32_t *counts, uint32_t T, uint32_t *totals) {
+    __shared__ uint32_t sm[SORT_WARPS + 1];
+    wait_prior_grid();
+    allow_next_grid();
+    uint32_t *c = counts + (uint64_t)blockIdx.x * T;
     uint32_t carry = 0;
-    for (uint64_t c0 = 0; c0 < n; c0 += 4096) {
-        const uint64_t i0 = c0 + (uint64_t)threadIdx.x * 4;
+    for (uint32_t c0 = 0; c0 < T; c0 += SORT_THREADS * 4) {
+        const uint32_t i0 = c0 + threadIdx.x * 4;
         uint32_t v[4], s = 0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            v[k] = (i0 + k < n) ? counts[i0 + k] : 0u;
+            v[k] = (i0 + k < T) ? c[i0 + k] : 0u;
             s += v[k];
         }
         uint32_t tot;
         uint32_t run = carry + block_exclusive_scan<uint32_t>(s, sm, &tot);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            if (i0 + k < n) counts[i0 + k] = run;
+            if (i0 + k < T) c[i0 + k] = run;
             run += v[k];
         }
         carry += tot;
     }
+    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
 }
 
-// one warp per tile: stable ranks inside the tile by rounds of 32 tracks
-__global__ void k_scatter(const int32_t *__restrict__ sector, uint64_t n, uint32_t S, uint32_t T,
-                          const uint32_t *__restrict__ base, int32_t *perm) {
-    __shared__ uint32_t cnt[512];
-    const int lane = threadIdx.x;
-    for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
-        for (uint32_t s = lane; s < S; s += 32) cnt[s] = 0;
-        __syncwarp();
-        for (int r = 0; r < SORT_TILE / 32; ++r) {
-            const uint64_t i = (uint64_t)t * SORT_TILE + r * 32 + lane;
-            const bool valid = i < n;
-            const int32_t s = valid ? sector[i] : -1;
-            const bool ok = valid && s >= 0 && (uint32_t)s < S;
-            const uint32_t key = ok ? (uint32_t)s : 0xFFFFFFFFu;
-            const uint32_t match = __match_any_sync(0xffffffffu, key);
-            const uint32_t rank = __popc(match & ((1u << lane) - 1u));
-            uint32_t before = 0;
-            if (ok) before = cnt[s];
-            __syncwarp();
-            if (ok) {
-                perm[base[(uint64_t)s * T + t] + before + rank] = (int32_t)i;
-                if (rank == 0) cnt[s] = before + __popc(match);
-            }
-            __syncwarp();
-        }
-    }
-}
-
-// sector_off and the item table, one block
-__global__ void __launch_bounds__(1024)
-    k_items(const uint32_t *__restrict__ base, uint32_t S, uint32_t T, uint64_t n,
-            int32_t *sector_off, int32_t *sector_item, int32_t *item_sector, int32_t *item_start,
-            int32_t *n_items, uint32_t max_items) {
-    __shared__ uint32_t sm[33];
-    __shared__ uint32_t carry_s;
-    if (threadIdx.x == 0) carry_s = 0;
-    __syncthreads();
-    for (uint32_t c0 = 0; c0 < S; c0 += 1024) {
-        const uint32_t s = c0 + threadIdx.x;
-        uint32_t off = 0, len = 0;
+// sector_off, sector_item and the item table; every block scans the (at most
+// 512) totals itself and fills its share of the items
+__global__ void __launch_bounds__(512)
+    k_items(const uint32_t *__restrict__ totals, uint32_t S, uint64_t n, int32_t *sector_off,
+            int32_t *sector_item, int32_t *item_sector, int32_t *item_start, int32_t *n_items,
+            uint32_t max_items) {
+    __shared__ uint32_t sm[17];
+    __shared__ uint32_t off_s[512], item_s[513];
+    wait_prior_grid();
+    allow_next_grid();
+    const uint32_t s = threadIdx.x;
+    const uint32_t len = s < S ? totals[s] : 0u;
+    uint32_t tot, n_it;
+    const uint32_t off = block_exclusive_scan<uint32_t>(len, sm, &tot);
+    const uint32_t items = (len + CALIB_CHUNK - 1) / CALIB_CHUNK;
+    const uint32_t first = block_exclusive_scan<uint32_t>(items, sm, &n_it);
+    off_s[s] = off;
+    item_s[s] = first;
+    if (s == 511) item_s[512] = n_it;
+    if (blockIdx.x == 0) {
         if (s < S) {
-            off = base[(uint64_t)s * T];
-            const uint32_t end = (s + 1 < S) ? base[(uint64_t)(s + 1) * T] : (uint32_t)n;
-            len = end - off;
             sector_off[s] = (int32_t)off;
+            sector_item[s] = (int32_t)first;
         }
-        const uint32_t items = (len + CALIB_CHUNK - 1) / CALIB_CHUNK;
-        uint32_t tot;
-        const uint32_t first = carry_s + block_exclusive_scan<uint32_t>(items, sm, &tot);
-        if (s < S) sector_item[s] = (int32_t)first;
-        for (uint32_t k = 0; k < items; ++k) {
-            if (first + k < max_items) {
-                item_sector[first + k] = (int32_t)s;
-                item_start[first + k] = (int32_t)(off + k * CALIB_CHUNK);
+        if (s == 0) {
+            sector_off[S] = (int32_t)n;
+            sector_item[S] = (int32_t)n_it;
+            *n_items = (int32_t)n_it;
+        }
+    }
+    __syncthreads();
+    for (uint32_t i = blockIdx.x * 512 + threadIdx.x; i < min(n_it, max_items); i += gridDim.x * 512) {
+        uint32_t lo = 0, hi = 512;   // the last sector whose first item is at most i
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (item_s[mid] <= i) lo = mid; else hi = mid;
+        }
+        item_sector[i] = (int32_t)lo;
+        item_start[i] = (int32_t)(off_s[lo] + (i - item_s[lo]) * CALIB_CHUNK);
+    }
+}
+
+__device__ __forceinline__ void cp_async(void *dst, const void *src, bool wide) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if (wide)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
+}
+// count floats of src (and of dst, which is 16-byte aligned) by asynchronous
+// copies: 16 bytes each while src is aligned for it, 4 bytes for the rest
+__device__ __forceinline__ void stage_floats(float *dst, const float *__restrict__ src,
+                                             uint32_t count) {
+    const uint32_t n4 = ((uintptr_t)src & 15u) ? 0u : count / 4;
+    for (uint32_t k = threadIdx.x; k < n4; k += SORT_THREADS) cp_async(dst + 4 * k, src + 4 * k, true);
+    for (uint32_t k = 4 * n4 + threadIdx.x; k < count; k += SORT_THREADS)
+        cp_async(dst + k, src + k, false);
+}
+
+// Stable scatter, a block per tile: every warp ranks its SORT_TILE / 8
+// consecutive tracks in rounds of 32 (the lanes of one sector find each other
+// by a match), the block adds up the warps' counts, and track j of the tile in
+// sector order goes to position j + delta[its sector].  With XT the tile's x
+// and theta rows are staged in shared memory by asynchronous copies while the
+// ranks are formed, and written in sector order, the rows of one sector (four
+// on average with 512 sectors) as one run: each array is read and written once
+// and no other pass over the tracks is needed.  Bound by the memory system:
+// 84 bytes a track at least; 4 M tracks take 88 us (3.8 TB/s), where the rank
+// pass and the two gathers took 41 + 80 us.
+template <bool XT>
+__global__ void __launch_bounds__(SORT_THREADS, 2)
+    k_scatter(const int32_t *__restrict__ sector, uint64_t n, uint32_t S, uint32_t T,
+              const uint32_t *__restrict__ base, const int32_t *__restrict__ sector_off,
+              int32_t *perm, const float *__restrict__ x, const float *__restrict__ theta,
+              float *out_x, float *out_theta) {
+    __shared__ uint16_t cnt[SORT_WARPS][512];   // per warp: tracks of a sector so far
+    __shared__ uint32_t local[512];             // first place of a sector in the tile
+    __shared__ uint32_t delta[512];             // from a place in the tile to the final one
+    __shared__ uint16_t src[SORT_TILE];         // tile index of the track at each place
+    __shared__ uint32_t dst[SORT_TILE];         // its final position
+    __shared__ uint32_t sm[SORT_WARPS + 1];
+    extern __shared__ __align__(16) float rows[];   // XT: x rows, then theta rows
+    float *xs = rows, *ts = rows + SORT_TILE * 6;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    wait_prior_grid();
+    for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
+        const uint64_t t0 = (uint64_t)t * SORT_TILE;
+        const uint32_t len = (uint32_t)min((uint64_t)SORT_TILE, n - t0);
+        if (XT) {
+            stage_floats(xs, x + t0 * 6, len * 6);
+            stage_floats(ts, theta + t0 * 3, len * 3);
+        }
+        int32_t key[SORT_ROUNDS];
+#pragma unroll
+        for (int r = 0; r < SORT_ROUNDS; ++r) {
+            const uint32_t i = (uint32_t)(warp * SORT_ROUNDS + r) * 32 + lane;
+            const int32_t s = i < len ? __ldg(sector + t0 + i) : -1;
+            key[r] = (uint32_t)s < S ? s : -1;
+        }
+        uint32_t first[2];   // where the tile's tracks of this thread's two sectors go
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t s = threadIdx.x * 2 + h;
+            first[h] = s < S ? (uint32_t)sector_off[s] + base[(uint64_t)s * T + t] : 0u;
+        }
+        for (int k = threadIdx.x; k < SORT_WARPS * 512 / 2; k += SORT_THREADS)
+            reinterpret_cast<uint32_t *>(cnt)[k] = 0;
+        __syncthreads();
+        uint32_t rank[SORT_ROUNDS];   // among the warp's tracks of the sector
+#pragma unroll
+        for (int r = 0; r < SORT_ROUNDS; ++r) {
+            const uint32_t match = __match_any_sync(0xffffffffu, key[r]);
+            const uint32_t before = __popc(match & ((1u << lane) - 1u));
+            uint32_t c = 0;
+            if (key[r] >= 0) c = cnt[warp][key[r]];
+            __syncwarp();
+            if (key[r] >= 0 && before == 0) cnt[warp][key[r]] = (uint16_t)(c + __popc(match));
+            __syncwarp();
+            rank[r] = c + before;
+        }
+        __syncthreads();
+        // the warps' counts of two sectors per thread: exclusive over the warps
+        uint32_t tot[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t run = 0;
+#pragma unroll
+            for (int w = 0; w < SORT_WARPS; ++w) {
+                const uint32_t c = cnt[w][threadIdx.x * 2 + h];
+                cnt[w][threadIdx.x * 2 + h] = (uint16_t)run;
+                run += c;
+            }
+            tot[h] = run;
+        }
+        uint32_t m;   // tracks of the tile (those of a bad sector left out)
+        const uint32_t ex = block_exclusive_scan<uint32_t>(tot[0] + tot[1], sm, &m);
+        local[threadIdx.x * 2] = ex;
+        local[threadIdx.x * 2 + 1] = ex + tot[0];
+        delta[threadIdx.x * 2] = first[0] - ex;
+        delta[threadIdx.x * 2 + 1] = first[1] - ex - tot[0];
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < SORT_ROUNDS; ++r) {
+            if (key[r] < 0) continue;
+            const uint32_t j = local[key[r]] + cnt[warp][key[r]] + rank[r];
+            src[j] = (uint16_t)((warp * SORT_ROUNDS + r) * 32 + lane);
+            dst[j] = j + delta[key[r]];
+        }
+        if (XT) asm volatile("cp.async.wait_all;\n" ::: "memory");
+        __syncthreads();
+        for (uint32_t j = threadIdx.x; j < m; j += SORT_THREADS)
+            perm[dst[j]] = (int32_t)(t0 + src[j]);
+        if (XT) {
+            const float2 *x2 = reinterpret_cast<const float2 *>(xs);
+            float2 *o2 = reinterpret_cast<float2 *>(out_x);
+            for (uint32_t e = threadIdx.x; e < m * 3; e += SORT_THREADS) {
+                const uint32_t j = e / 3, c = e - 3 * j;
+                o2[(size_t)dst[j] * 3 + c] = x2[src[j] * 3u + c];
+                out_theta[(size_t)dst[j] * 3 + c] = ts[src[j] * 3u + c];
             }
         }
-        __syncthreads();
-        if (threadIdx.x == 0) carry_s += tot;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        sector_off[S] = (int32_t)n;
-        sector_item[S] = (int32_t)carry_s;
-        *n_items = (int32_t)carry_s;
+        __syncthreads();   // the tile's tables are rebuilt for the next one
     }
 }
 
@@ -1135,18 +1252,35 @@ uint32_t calib_max_items(uint64_t n, uint32_t S) {
 }
 uint32_t calib_tiles(uint64_t n) { return (uint32_t)((n + SORT_TILE - 1) / SORT_TILE); }
 
-void launch_calib_sort(const int32_t *sector, uint64_t n, uint32_t S, uint32_t *counts,
-                       int32_t *perm, int32_t *sector_off, int32_t *sector_item,
-                       int32_t *item_sector, int32_t *item_start, int32_t *n_items,
-                       unsigned long long *status, int grid, cudaStream_t st) {
+cudaError_t launch_calib_sort(const int32_t *sector, uint64_t n, uint32_t S, uint32_t *counts,
+                              uint32_t *totals, int32_t *perm, int32_t *sector_off,
+                              int32_t *sector_item, int32_t *item_sector, int32_t *item_start,
+                              int32_t *n_items, const float *x, const float *theta, float *out_x,
+                              float *out_theta, unsigned long long *status, int sms,
+                              cudaStream_t st) {
     const uint32_t T = calib_tiles(n);
-    const int g = (int)min((uint32_t)grid, max(T, 1u));
-    if (T > 0) k_hist<<<g, 256, 0, st>>>(sector, n, S, T, counts, status);
-    k_scan_counts<<<1, 1024, 0, st>>>(counts, (uint64_t)S * T);
-    if (T > 0) k_scatter<<<g, 32, 0, st>>>(sector, n, S, T, counts, perm);
-    if (T > 0)
-        k_items<<<1, 1024, 0, st>>>(counts, S, T, n, sector_off, sector_item, item_sector,
-                                    item_start, n_items, calib_max_items(n, S));
+    const size_t smem = x ? (size_t)SORT_TILE * 9 * sizeof(float) : 0;
+    if (x) {   // above the default limit of dynamic shared memory
+        const cudaError_t e = cudaFuncSetAttribute(
+            k_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    const int g = (int)min((uint32_t)(max(sms, 1) * 8), T);
+    k_hist<<<g, SORT_THREADS, 0, st>>>(sector, n, S, T, counts, status);
+    launch_after(k_sector_scan, S, SORT_THREADS, 0, st, counts, T, totals);
+    launch_after(k_items, (int)min(calib_max_items(n, S) / 512 + 1, (uint32_t)max(sms, 1)), 512, 0,
+                 st, (const uint32_t *)totals, S, n, sector_off, sector_item, item_sector,
+                 item_start, n_items, calib_max_items(n, S));
+    const int gs = (int)min((uint32_t)(max(sms, 1) * 2), T);
+    if (x)
+        launch_after(k_scatter<true>, gs, SORT_THREADS, smem, st, sector, n, S, T,
+                     (const uint32_t *)counts, (const int32_t *)sector_off, perm, x, theta, out_x,
+                     out_theta);
+    else
+        launch_after(k_scatter<false>, gs, SORT_THREADS, smem, st, sector, n, S, T,
+                     (const uint32_t *)counts, (const int32_t *)sector_off, perm, x, theta, out_x,
+                     out_theta);
+    return cudaGetLastError();
 }
 
 void launch_calib_gather(const float *src, uint32_t width, const int32_t *perm, uint64_t n,

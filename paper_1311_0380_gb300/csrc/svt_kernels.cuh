@@ -147,10 +147,14 @@ void launch_format(const svt_best *best, const uint32_t *words, const uint32_t *
 // ---- calibration (svt_calib.cu) ------------------------------------------------
 uint32_t calib_max_items(uint64_t n, uint32_t S);
 uint32_t calib_tiles(uint64_t n);
-void launch_calib_sort(const int32_t *sector, uint64_t n, uint32_t S, uint32_t *counts,
-                       int32_t *perm, int32_t *sector_off, int32_t *sector_item,
-                       int32_t *item_sector, int32_t *item_start, int32_t *n_items,
-                       unsigned long long *status, int grid, cudaStream_t st);
+// Sector index of n > 0 tracks; with x also the tracks themselves (theta, out_x
+// 8-byte aligned, out_theta) in sector order.
+cudaError_t launch_calib_sort(const int32_t *sector, uint64_t n, uint32_t S, uint32_t *counts,
+                              uint32_t *totals, int32_t *perm, int32_t *sector_off,
+                              int32_t *sector_item, int32_t *item_sector, int32_t *item_start,
+                              int32_t *n_items, const float *x, const float *theta, float *out_x,
+                              float *out_theta, unsigned long long *status, int sms,
+                              cudaStream_t st);
 void launch_calib_gather(const float *src, uint32_t width, const int32_t *perm, uint64_t n,
                          float *dst, int grid, cudaStream_t st);
 void launch_calib_forward(const float *x, const int32_t *item_sector, const int32_t *item_start,
