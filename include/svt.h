@@ -257,8 +257,7 @@ int svt_fit(const uint32_t *d_words, const uint32_t *d_road_word, const uint32_t
 
 /*
  * svt_select -- chi-square cut and best combination per road (one warp per
- * road, shuffle argmin; roads of more than 4096 combinations one block each,
- * in a second launch).
+ * road; roads of more than 1024 combinations one block each).
  *   d_fit_chi2, d_fit_par, comb_cap   from svt_fit
  *   d_comb_off, d_road_flags          from svt_combine
  *   d_best[road_cap]       out: per-road best (svt_best)

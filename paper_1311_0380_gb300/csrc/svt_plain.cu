@@ -3,7 +3,9 @@
 // the best passing combination per road, format packs the records.  This is
 // the structure of the paper's Sec. 2.1 GPU port (one kernel per stage, the
 // loops unrolled so that one thread handles one combination), kept here as
-// the baseline of the fused path and as the per-stage C ABI.
+// the baseline of the fused path and as the per-stage C ABI.  Its launches are
+// chained like the fused path's (launch_after): each kernel waits for the one
+// before it on the device, so the gaps between the eight short launches overlap.
 #include "svt_kernels.cuh"
 
 namespace svt {
@@ -19,6 +21,8 @@ __global__ void k_combine_count(const uint32_t *__restrict__ road_nhit,
                                 const uint64_t *__restrict__ n_roads, uint64_t road_cap,
                                 const svt_config cfg, uint32_t *road_flags, uint64_t *comb_cnt,
                                 const unsigned long long *status) {
+    wait_prior_grid();
+    allow_next_grid();
     if (!status_ok(status)) return;
     const uint64_t R = road_count(n_roads, road_cap);
     for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < R;
@@ -47,6 +51,8 @@ __global__ void __launch_bounds__(SCAN_THREADS)
     k_scan_u64_reduce(const uint64_t *__restrict__ a, const uint64_t *__restrict__ n_dev,
                       uint64_t cap, uint64_t *tile_sums, const unsigned long long *status) {
     __shared__ unsigned long long red[SCAN_THREADS / 32 + 1];
+    wait_prior_grid();
+    allow_next_grid();
     if (!status_ok(status)) return;
     const uint64_t n = *n_dev < cap ? *n_dev : cap;
     const uint64_t T = (n + SCAN_TILE - 1) / SCAN_TILE;
@@ -65,6 +71,8 @@ __global__ void __launch_bounds__(1024)
     k_scan_u64_tiles(uint64_t *tile_sums, const uint64_t *__restrict__ n_dev, uint64_t cap,
                      const unsigned long long *status) {
     __shared__ unsigned long long sm[33];
+    wait_prior_grid();
+    allow_next_grid();
     if (!status_ok(status)) return;
     const uint64_t n = *n_dev < cap ? *n_dev : cap;
     const uint64_t T = (n + SCAN_TILE - 1) / SCAN_TILE;
@@ -85,6 +93,8 @@ __global__ void __launch_bounds__(SCAN_THREADS)
                      const uint64_t *__restrict__ tile_sums, uint64_t *total,
                      const unsigned long long *status) {
     __shared__ unsigned long long red[SCAN_THREADS / 32 + 1];
+    wait_prior_grid();
+    allow_next_grid();
     if (!status_ok(status)) return;
     const uint64_t n = *n_dev < cap ? *n_dev : cap;
     const uint64_t T = (n + SCAN_TILE - 1) / SCAN_TILE;
@@ -110,169 +120,162 @@ __global__ void __launch_bounds__(SCAN_THREADS)
     }
 }
 
-// Roads with more combinations than this are written (combine) and scanned
-// (select) by a whole block in a second launch, so that one long road does
-// not hold up a warp while the others have finished.
-constexpr uint64_t PLAIN_BIG = 4096;
-
-// Per-road metadata for the plain combine and select, read for a group of
-// roads at once (one coalesced load per field) instead of road by road.
+// Per-road metadata of the plain select, read for a group of roads at once
+// (one coalesced load per field) instead of road by road.
 struct RoadMeta {
     uint64_t off, n;
-    uint32_t word;   // road_nhit (combine) or road_flags (select)
+    uint32_t word;   // road_flags
 };
 
-// Metadata of road r (zeros past the last road).
-__device__ __forceinline__ RoadMeta road_meta(const uint64_t *__restrict__ comb_off,
-                                              const uint32_t *__restrict__ word, uint64_t R,
-                                              uint64_t r) {
-    RoadMeta m{0, 0, 0};
-    if (r < R) {
-        m.off = __ldg(comb_off + r);
-        m.n = __ldg(comb_off + r + 1) - m.off;
-        m.word = __ldg(word + r);
+// Every combination of every road, written in order by tiles of WRITE_TILE
+// consecutive combinations: thread t of a block takes WRITE_PER consecutive
+// ones, finds the road of its first (a search of the tile's offsets, staged in
+// shared memory), derives that combination's digits once by
+// division and counts them up from there (see the counter below), taking up the next
+// road where one ends.  The tiles are equal work whatever the roads' sizes (a
+// road per warp, or per block for big ones, left the largest roads running
+// alone: 95 us of the scaled workload's 200 events against 26 us), and each
+// thread's two runs of 32 bytes leave as 16-byte stores.  The tile's roads are
+// found by 32-way searches, three dependent loads where a binary search of the
+// 12,800 offsets makes fourteen, and the digits cost about sixteen instructions a
+// combination (34 us with binary searches and digits counted one by one).
+constexpr int WRITE_THREADS = 256, WRITE_PER = 8, WRITE_TILE = WRITE_THREADS * WRITE_PER;
+constexpr uint32_t WRITE_ROADS = 512;   // staged roads of a tile; more are searched in place
+
+// largest r in [lo, hi) with off[r] <= j, given off[lo] <= j: the last of
+// several roads at one offset, which is the one that has combinations
+__device__ __forceinline__ uint64_t road_of(const uint64_t *off, uint64_t lo, uint64_t hi,
+                                            uint64_t j) {
+    while (hi - lo > 1) {
+        const uint64_t mid = (lo + hi) >> 1;
+        if (off[mid] <= j) lo = mid; else hi = mid;
     }
-    return m;
+    return lo;
+}
+// the same by a warp, 32 offsets a step
+__device__ __forceinline__ uint64_t road_of_warp(const uint64_t *__restrict__ off, uint64_t lo,
+                                                 uint64_t hi, uint64_t j, uint32_t lane) {
+    while (hi - lo > 1) {
+        const uint64_t step = (hi - lo + 31) / 32, p = lo + lane * step;
+        const uint32_t le = __ballot_sync(0xffffffffu, p < hi && __ldg(off + p) <= j);
+        lo += (31u - __clz(le)) * step;   // lane 0's is always set
+        hi = min(lo + step, hi);
+    }
+    return lo;
 }
 
-// Big roads of a block's group of blockDim.x roads, compacted into `list`
-// (their metadata and index); returns how many (a block-wide call).
-__device__ __forceinline__ uint32_t big_roads_of_group(const RoadMeta &mine, uint64_t r,
-                                                       bool big, RoadMeta *list,
-                                                       uint32_t *list_r, uint32_t *count) {
-    if (threadIdx.x == 0) *count = 0;
-    __syncthreads();
-    if (big) {
-        const uint32_t k = atomicAdd(count, 1u);
-        list[k] = mine;
-        list_r[k] = (uint32_t)r;
-    }
-    __syncthreads();
-    return *count;
+// 16 - n'_l of every layer, layer 5 in the lowest four bits (0 for 16 hits)
+__device__ __forceinline__ uint32_t digit_bias(const RoadShape &s) {
+    uint32_t b = 0;
+#pragma unroll
+    for (int l = 0; l < N_LAYERS; ++l) b |= ((16u - s.n[l]) & 15u) << (4 * (N_LAYERS - 1 - l));
+    return b;
 }
 
-// Rows [a_begin, a_end) of one road's combinations in index order
-// c = a * NB + b, with the layers split as in the fused path (road_split: a
-// suffix of at least 32 combinations gives the column b, the prefix the row
-// a).  A lane derives the suffix digits of its column once per pass over the
-// columns; the prefix digits (the same for all lanes) are derived for the
-// first row and then counted up row by row (layer split-1 fastest, a carry
-// only when a digit wraps), so a combination costs a few instructions and
-// two coalesced stores.
-__device__ __forceinline__ void write_rows(uint32_t r, const RoadMeta &m, const RoadShape &s,
-                                           uint32_t split, uint32_t NB, uint32_t a_begin,
-                                           uint32_t a_end, uint32_t xft_pairs, int lane,
-                                           uint32_t *comb_road, uint32_t *comb_hits) {
-    uint32_t mg[N_LAYERS], top = 0;   // top: n'_l - 1 of every layer, 4 bits each
-#pragma unroll
-    for (int l = 0; l < N_LAYERS; ++l) {
-        mg[l] = kDivMagic[s.n[l]];
-        top |= (s.n[l] - 1u) << (4 * l);
-    }
-    uint32_t ra = a_begin, pa0 = 0;   // prefix digits of the first row
-#pragma unroll
-    for (int l = N_LAYERS - 1; l >= 0; --l) {
-        if ((uint32_t)l < split) {
-            const uint32_t qd = div_by(ra, s.n[l], mg[l]);
-            pa0 |= (ra - qd * s.n[l]) << (4 * l);
-            ra = qd;
-        }
-    }
-    for (uint32_t b0 = 0; b0 < NB; b0 += 32) {
-        const uint32_t b = b0 + (uint32_t)lane;
-        uint32_t rem = b, pb = 0;   // digits of the suffix layers split..5
-#pragma unroll
-        for (int l = N_LAYERS - 1; l >= 0; --l) {
-            if ((uint32_t)l >= split) {
-                const uint32_t qd = div_by(rem, s.n[l], mg[l]);
-                pb |= (rem - qd * s.n[l]) << (4 * l);
-                rem = qd;
-            }
-        }
-        uint32_t pa = pa0;
-        uint64_t c = (uint64_t)a_begin * NB + b;
-        for (uint32_t a = a_begin; a < a_end; ++a, c += NB) {
-            if (b < NB && c < m.n) {
-                uint32_t packed = pa | pb;
-                if (xft_pairs) packed |= ((packed >> 16) & 15u) << 20;   // layer 5 takes layer 4's hit
-                comb_road[m.off + c] = r;
-                comb_hits[m.off + c] = packed;
-            }
-            for (int l = (int)split - 1; l >= 0; --l) {   // next row
-                const uint32_t sh = 4u * (uint32_t)l;
-                if (((pa >> sh) & 15u) != ((top >> sh) & 15u)) {
-                    pa += 1u << sh;
-                    break;
-                }
-                pa &= ~(15u << sh);
-            }
-        }
-    }
-}
-
-// A road per warp (roads of at most PLAIN_BIG combinations, each combination's
-// digits by division; the next road's entries are read while this one is
-// written), or a big road per block whose eight warps take one block of rows
-// each (write_rows).
-template <bool BIG>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(WRITE_THREADS)
     k_combine_write(const uint32_t *__restrict__ road_nhit, const uint64_t *__restrict__ n_roads,
                     uint64_t road_cap, const uint64_t *__restrict__ comb_off, uint64_t comb_cap,
                     uint32_t xft_pairs, uint32_t *comb_road, uint32_t *comb_hits,
                     unsigned long long *status) {
-    __shared__ RoadMeta list[256];
-    __shared__ uint32_t list_r[256], list_n;
+    __shared__ uint64_t ends[2];   // roads of the tile's first and last combination
+    __shared__ uint64_t off_s[WRITE_ROADS + 1];
+    __shared__ uint32_t nhit_s[WRITE_ROADS];
+    wait_prior_grid();
+    allow_next_grid();
     if (!status_ok(status)) return;
     const uint64_t R = road_count(n_roads, road_cap);
-    const int lane = threadIdx.x & 31;
-    const uint64_t warp0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    if (!BIG && warp0 == 0 && lane == 0 && comb_off[R] > comb_cap) report(status, 0, SVT_ERR_OOM);
-    if (!BIG) {
-        RoadMeta m = road_meta(comb_off, road_nhit, R, warp0);
-        for (uint64_t r = warp0; r < R; r += n_warps) {
-            const RoadMeta next = road_meta(comb_off, road_nhit, R, r + n_warps);
-            if (m.n && m.n <= PLAIN_BIG && m.off + m.n <= comb_cap) {
-                const RoadShape s = road_shape(m.word, xft_pairs);
-                uint32_t mg[N_LAYERS];
+    const uint64_t total = comb_off[R];
+    if (total > comb_cap) {   // nothing to write: the status says so
+        if (blockIdx.x == 0 && threadIdx.x == 0) report(status, 0, SVT_ERR_OOM);
+        return;
+    }
+    const bool wide = (((uintptr_t)comb_road | (uintptr_t)comb_hits) & 15u) == 0;
+    for (uint64_t t0 = (uint64_t)blockIdx.x * WRITE_TILE; t0 < total;
+         t0 += (uint64_t)gridDim.x * WRITE_TILE) {
+        const uint64_t t1 = min(t0 + (uint64_t)WRITE_TILE, total);
+        if (threadIdx.x < 64) {
+            const uint64_t r = road_of_warp(comb_off, 0, R, threadIdx.x < 32 ? t0 : t1 - 1,
+                                            threadIdx.x & 31u);
+            if ((threadIdx.x & 31u) == 0) ends[threadIdx.x >> 5] = r;
+        }
+        __syncthreads();
+        const uint64_t r0 = ends[0], nr = ends[1] - r0 + 1;
+        const bool staged = nr <= WRITE_ROADS;
+        if (staged) {
+            for (uint64_t k = threadIdx.x; k <= nr; k += WRITE_THREADS) {
+                off_s[k] = __ldg(comb_off + r0 + k);
+                if (k < nr) nhit_s[k] = __ldg(road_nhit + r0 + k);
+            }
+            __syncthreads();
+        }
+        // offsets and hits of the tile's roads, by their place from r0
+        const uint64_t *off = staged ? off_s : comb_off + r0;
+        const uint32_t *nhit = staged ? nhit_s : road_nhit + r0;
+        const uint64_t j0 = t0 + (uint64_t)threadIdx.x * WRITE_PER;
+        if (j0 < t1) {
+            uint64_t r = road_of(off, 0, nr, j0);
+            RoadShape s = road_shape(nhit[r], xft_pairs);
+            uint64_t end = off[r + 1];
+            // The digits as a counter with layer 5 in the lowest four bits, each
+            // raised by 16 - n'_l, so that a digit past its layer's last hit carries
+            // into the next slower layer by itself and leaves zero, which no raised
+            // digit is (unless n'_l = 16, where nothing has to be put back).
+            uint32_t rem = (uint32_t)(j0 - off[r]), x = 0, bias = digit_bias(s);
 #pragma unroll
-                for (int l = 0; l < N_LAYERS; ++l) mg[l] = kDivMagic[s.n[l]];
-                for (uint64_t c = lane; c < m.n; c += 32) {
-                    uint32_t rem = (uint32_t)c, packed = 0;
+            for (int l = N_LAYERS - 1; l >= 0; --l) {
+                const uint32_t qd = div_by(rem, s.n[l], kDivMagic[s.n[l]]);
+                x |= (rem - qd * s.n[l]) << (4 * (N_LAYERS - 1 - l));
+                rem = qd;
+            }
+            x += bias;
+            // combinations up to the road's end (the last of them resets the counter)
+            uint32_t left = (uint32_t)min(end - j0, (uint64_t)WRITE_PER + 1);
+            uint32_t road[WRITE_PER], hits[WRITE_PER];
 #pragma unroll
-                    for (int l = N_LAYERS - 1; l >= 0; --l) {
-                        const uint32_t qd = div_by(rem, s.n[l], mg[l]);
-                        packed |= (rem - qd * s.n[l]) << (4 * l);
-                        rem = qd;
+            for (int i = 0; i < WRITE_PER; ++i) {
+                road[i] = (uint32_t)(r0 + r);
+                // layer 0 to the lowest bits: the nibbles of each byte and the
+                // three bytes change places
+                const uint32_t d = x - bias;
+                const uint32_t sw = ((d >> 4) & 0x0F0F0Fu) | ((d << 4) & 0xF0F0F0u);
+                const uint32_t h = __byte_perm(sw, 0u, 0x4012);
+                // with pairs layer 5 (radix 1) takes layer 4's hit
+                hits[i] = xft_pairs ? h | (((h >> 16) & 15u) << 20) : h;
+                if (--left == 0) {   // the next road that has combinations
+                    if (j0 + i + 1 < t1) {
+                        do {
+                            ++r;
+                            end = off[r + 1];
+                        } while (end == j0 + i + 1);
+                        s = road_shape(nhit[r], xft_pairs);
+                        bias = digit_bias(s);
+                        left = (uint32_t)min(end - (j0 + i + 1), (uint64_t)WRITE_PER + 1);
                     }
-                    if (xft_pairs) packed |= ((packed >> 16) & 15u) << 20;
-                    comb_road[m.off + c] = (uint32_t)r;
-                    comb_hits[m.off + c] = packed;
+                    x = bias;
+                } else {
+                    x += 1u;
+                    const uint32_t z = ~(x | (x >> 1) | (x >> 2) | (x >> 3)) & 0x111111u;
+                    x += bias & (z * 15u);
                 }
             }
-            m = next;
-        }
-    } else {
-        const uint32_t warp = threadIdx.x >> 5, n_w = blockDim.x >> 5;
-        for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x; g < R;
-             g += (uint64_t)gridDim.x * blockDim.x) {
-            const uint64_t r = g + threadIdx.x;
-            const RoadMeta mine = road_meta(comb_off, road_nhit, R, r);
-            const bool big = mine.n > PLAIN_BIG && mine.off + mine.n <= comb_cap;
-            const uint32_t nb = big_roads_of_group(mine, r, big, list, list_r, &list_n);
-            for (uint32_t k = 0; k < nb; ++k) {
-                const RoadMeta m = list[k];
-                const RoadShape s = road_shape(m.word, xft_pairs);
-                uint32_t split, NB;
-                road_split(s, split, NB);
-                const uint32_t NA = (uint32_t)((m.n + NB - 1) / NB);
-                const uint32_t per = (NA + n_w - 1) / n_w;
-                const uint32_t a0 = min(warp * per, NA), a1 = min(a0 + per, NA);
-                write_rows(list_r[k], m, s, split, NB, a0, a1, xft_pairs, lane, comb_road,
-                           comb_hits);
+            if (wide && j0 + WRITE_PER <= t1) {
+#pragma unroll
+                for (int i = 0; i < WRITE_PER; i += 4) {
+                    *reinterpret_cast<uint4 *>(comb_road + j0 + i) =
+                        make_uint4(road[i], road[i + 1], road[i + 2], road[i + 3]);
+                    *reinterpret_cast<uint4 *>(comb_hits + j0 + i) =
+                        make_uint4(hits[i], hits[i + 1], hits[i + 2], hits[i + 3]);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < WRITE_PER; ++i)
+                    if (j0 + i < t1) {
+                        comb_road[j0 + i] = road[i];
+                        comb_hits[j0 + i] = hits[i];
+                    }
             }
-            __syncthreads();   // the list is rebuilt for the next group
         }
+        __syncthreads();   // `ends` is set again for the next tile
     }
 }
 
@@ -398,6 +401,8 @@ __global__ void __launch_bounds__(FIT_THREADS, 5)
     __shared__ StagedRow rows[FIT_STAGE_ROADS];
     __shared__ uint16_t coords[FIT_STAGE_ROADS][N_LAYERS * MAX_HITS];
     __shared__ uint32_t tile_r0, tile_nr;
+    wait_prior_grid();
+    allow_next_grid();
     if (!status_ok(status)) return;
     const uint64_t n = *n_combs < comb_cap ? *n_combs : comb_cap;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -470,116 +475,119 @@ __global__ void __launch_bounds__(FIT_THREADS, 5)
     }
 }
 
-// Best passing combination of road r from its chi2 values, over the threads
-// [idx, idx + step, ...) of the warp (step 32) or block (step 256): each
-// visits its combinations in increasing c (a block keeps eight loads per
-// thread in flight), so a strict '<' keeps the smallest index among equal chi2; the
-// (chi2, c) keys are then merged (over the block through red, when BIG).
-// Written by thread idx 0.
-template <bool BIG>
-__device__ __forceinline__ void select_road(uint32_t r, const RoadMeta &m,
-                                            const uint32_t *__restrict__ fit_chi2,
-                                            const int32_t *__restrict__ fit_par,
-                                            uint64_t comb_cap, uint32_t init_chi, uint32_t idx,
-                                            uint32_t step, int lane, unsigned long long *red,
-                                            svt_best *best) {
+// Best passing combination of a road from its chi2 values, over the threads
+// idx, idx + STEP, ... (a warp, or the block): each visits its combinations in
+// increasing c, sixteen loads in flight, so a strict '<' keeps the smallest
+// index among equal chi2.  Returns this thread's key (chi2 << 32) | c.
+template <uint32_t STEP>
+__device__ __forceinline__ unsigned long long scan_chi2(const uint32_t *__restrict__ chi2,
+                                                        uint64_t n, uint32_t init_chi,
+                                                        uint32_t idx) {
+    constexpr int U = 16;
     uint32_t bchi = init_chi, bc = 0;
-    if (!BIG && m.off + m.n <= comb_cap) {
-        for (uint64_t c = idx; c < m.n; c += step) {
-            const uint32_t v = __ldg(fit_chi2 + m.off + c);
-            if (v < bchi) {
-                bchi = v;
-                bc = (uint32_t)c;
+    for (uint64_t c0 = idx; c0 < n; c0 += (uint64_t)U * STEP) {
+        uint32_t v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t c = c0 + (uint64_t)u * STEP;
+            v[u] = c < n ? __ldg(chi2 + c) : 0xFFFFFFFFu;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (v[u] < bchi) {
+                bchi = v[u];
+                bc = (uint32_t)c0 + (uint32_t)u * STEP;
             }
-        }
-    } else if (m.off + m.n <= comb_cap) {
-        for (uint64_t c0 = idx; c0 < m.n; c0 += 8ull * step) {
-            uint32_t v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint64_t c = c0 + (uint64_t)u * step;
-                v[u] = c < m.n ? __ldg(fit_chi2 + m.off + c) : 0xFFFFFFFFu;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (v[u] < bchi) {
-                    bchi = v[u];
-                    bc = (uint32_t)(c0 + (uint64_t)u * step);
-                }
-        }
     }
-    unsigned long long key = bchi != init_chi ? (((unsigned long long)bchi << 32) | bc) : ~0ull;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        unsigned long long o = __shfl_xor_sync(0xffffffffu, key, d);
-        key = o < key ? o : key;
-    }
-    if (BIG) {
-        if (lane == 0) red[threadIdx.x >> 5] = key;
-        __syncthreads();
-        if (threadIdx.x == 0)
-            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) key = red[w] < key ? red[w] : key;
-        __syncthreads();   // red is reused by the next road
-    }
-    if (idx == 0) {
-        svt_best b;
-        b.flags = m.word;
-        if (key != ~0ull) {
-            const uint32_t c = (uint32_t)key;
-            b.flags |= SVT_FLAG_PASS;
-            b.comb = c;
-            b.chi2 = (uint32_t)(key >> 32);
-            b.p[0] = fit_par[m.off + c];
-            b.p[1] = fit_par[comb_cap + m.off + c];
-            b.p[2] = fit_par[2 * comb_cap + m.off + c];
-        } else {
-            b.comb = 0xFFFFFFFFu;
-            b.chi2 = 0;
-            b.p[0] = b.p[1] = b.p[2] = 0;
-        }
-        best[r] = b;
-    }
+    return bchi != init_chi ? (((unsigned long long)bchi << 32) | bc) : ~0ull;
 }
 
-// Chi-square cut and best combination of each road: a road per warp (roads of
-// at most PLAIN_BIG combinations), or a big road per block.
-template <bool BIG>
-__global__ void __launch_bounds__(256)
+__device__ __forceinline__ unsigned long long warp_min_key(unsigned long long key) {
+    const uint32_t hi = __reduce_min_sync(0xffffffffu, (uint32_t)(key >> 32));
+    const uint32_t lo = __reduce_min_sync(
+        0xffffffffu, (uint32_t)(key >> 32) == hi ? (uint32_t)key : 0xFFFFFFFFu);
+    return ((unsigned long long)hi << 32) | lo;
+}
+
+// Chi-square cut and best combination of each road.  A block takes
+// SELECT_GROUP consecutive roads at a time: its warps share those of at most
+// SELECT_BIG combinations, then the whole block scans each longer one.
+// Bound at the end by the longest road's block, hence the sixteen loads: with
+// eight the scaled workload's 200 events (12,800 roads, one of 100 thousand
+// combinations) take 33 us instead of 22; blocks of 512 or 1024 threads take 26
+// to 34, groups of 8 to 64 roads 22 to 32.  (Groups of 256 roads, and long roads
+// in a launch of their own, left most of the GPU waiting for a few blocks: 86 us.)
+constexpr uint32_t SELECT_THREADS = 256, SELECT_GROUP = 16, SELECT_BIG = 1024;
+__global__ void __launch_bounds__(SELECT_THREADS)
     k_select(const uint32_t *__restrict__ fit_chi2, const int32_t *__restrict__ fit_par,
              uint64_t comb_cap, const uint64_t *__restrict__ comb_off,
              const uint32_t *__restrict__ road_flags, const uint64_t *__restrict__ n_roads,
              uint64_t road_cap, const svt_config cfg, svt_best *best,
              const unsigned long long *status) {
-    __shared__ unsigned long long red[8];
-    __shared__ RoadMeta list[256];
-    __shared__ uint32_t list_r[256], list_n;
+    __shared__ RoadMeta meta[SELECT_GROUP];
+    __shared__ unsigned long long key_s[SELECT_GROUP];
+    __shared__ uint32_t next;
+    wait_prior_grid();
+    allow_next_grid();
     if (!status_ok(status)) return;
     const uint64_t R = road_count(n_roads, road_cap);
-    const int lane = threadIdx.x & 31;
-    const uint64_t warp0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const uint32_t lane = threadIdx.x & 31u;
     const uint32_t init_chi = cfg.chi2_cut == 0xFFFFFFFFu ? 0xFFFFFFFFu : cfg.chi2_cut + 1u;
-    if (!BIG) {
-        RoadMeta m = road_meta(comb_off, road_flags, R, warp0);
-        for (uint64_t r = warp0; r < R; r += n_warps) {
-            const RoadMeta next = road_meta(comb_off, road_flags, R, r + n_warps);
-            if (m.n <= PLAIN_BIG)
-                select_road<false>((uint32_t)r, m, fit_chi2, fit_par, comb_cap, init_chi,
-                                   (uint32_t)lane, 32u, lane, red, best);
-            m = next;
+    for (uint64_t g = (uint64_t)blockIdx.x * SELECT_GROUP; g < R;
+         g += (uint64_t)gridDim.x * SELECT_GROUP) {
+        const uint32_t n = (uint32_t)min((uint64_t)SELECT_GROUP, R - g);
+        if (threadIdx.x == 0) next = 0;
+        if (threadIdx.x < SELECT_GROUP) {
+            RoadMeta m{0, 0, 0};
+            if (threadIdx.x < n) {
+                m.off = __ldg(comb_off + g + threadIdx.x);
+                m.n = __ldg(comb_off + g + threadIdx.x + 1) - m.off;
+                m.word = __ldg(road_flags + g + threadIdx.x);
+                if (m.off + m.n > comb_cap) m.n = 0;   // (an error status by now)
+            }
+            meta[threadIdx.x] = m;
+            key_s[threadIdx.x] = ~0ull;
         }
-    } else {
-        for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x; g < R;
-             g += (uint64_t)gridDim.x * blockDim.x) {
-            const uint64_t r = g + threadIdx.x;
-            const RoadMeta mine = road_meta(comb_off, road_flags, R, r);
-            const uint32_t nb = big_roads_of_group(mine, r, mine.n > PLAIN_BIG, list, list_r,
-                                                   &list_n);
-            for (uint32_t k = 0; k < nb; ++k)
-                select_road<true>(list_r[k], list[k], fit_chi2, fit_par, comb_cap, init_chi,
-                                  threadIdx.x, blockDim.x, lane, red, best);
-            __syncthreads();   // the list is rebuilt for the next group
+        __syncthreads();
+        for (;;) {
+            uint32_t k = 0;
+            if (lane == 0) k = atomicAdd(&next, 1u);
+            k = __shfl_sync(0xffffffffu, k, 0);
+            if (k >= n) break;
+            const RoadMeta m = meta[k];
+            if (m.n == 0 || m.n > SELECT_BIG) continue;
+            const unsigned long long key =
+                warp_min_key(scan_chi2<32>(fit_chi2 + m.off, m.n, init_chi, lane));
+            if (lane == 0) key_s[k] = key;
         }
+        for (uint32_t k = 0; k < n; ++k) {
+            const RoadMeta m = meta[k];
+            if (m.n <= SELECT_BIG) continue;   // uniform over the block
+            const unsigned long long key = warp_min_key(
+                scan_chi2<SELECT_THREADS>(fit_chi2 + m.off, m.n, init_chi, threadIdx.x));
+            if (lane == 0) atomicMin(&key_s[k], key);
+        }
+        __syncthreads();
+        if (threadIdx.x < n) {
+            const RoadMeta m = meta[threadIdx.x];
+            const unsigned long long key = key_s[threadIdx.x];
+            svt_best b;
+            b.flags = m.word;
+            b.comb = 0xFFFFFFFFu;
+            b.chi2 = 0;
+            b.p[0] = b.p[1] = b.p[2] = 0;
+            if (key != ~0ull) {
+                const uint32_t c = (uint32_t)key;
+                b.flags |= SVT_FLAG_PASS;
+                b.comb = c;
+                b.chi2 = (uint32_t)(key >> 32);
+                b.p[0] = fit_par[m.off + c];
+                b.p[1] = fit_par[comb_cap + m.off + c];
+                b.p[2] = fit_par[2 * comb_cap + m.off + c];
+            }
+            best[g + threadIdx.x] = b;
+        }
+        __syncthreads();   // the group's tables are rebuilt for the next one
     }
 }
 
@@ -587,6 +595,8 @@ __global__ void k_format(const svt_best *__restrict__ best, const uint32_t *__re
                          const uint32_t *__restrict__ road_word,
                          const uint64_t *__restrict__ n_roads, uint64_t road_cap, uint32_t *out,
                          const unsigned long long *status) {
+    wait_prior_grid();
+    allow_next_grid();
     if (!status_ok(status)) return;
     const uint64_t R = road_count(n_roads, road_cap);
     for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < R;
@@ -614,17 +624,18 @@ int grid_for(uint64_t n, int threads, int max_grid) {
 void launch_combine_count(const uint32_t *road_nhit, const uint64_t *n_roads, uint64_t road_cap,
                           const svt_config cfg, uint32_t *road_flags, uint64_t *comb_cnt,
                           const unsigned long long *status, int grid, cudaStream_t st) {
-    k_combine_count<<<grid_for(road_cap, 256, grid), 256, 0, st>>>(road_nhit, n_roads, road_cap,
-                                                                   cfg, road_flags, comb_cnt,
-                                                                   status);
+    launch_after(k_combine_count, grid_for(road_cap, 256, grid), 256, 0, st, road_nhit, n_roads,
+                 road_cap, cfg, road_flags, comb_cnt, status);
 }
 
 void launch_scan_u64(uint64_t *a, const uint64_t *n_dev, uint64_t cap, uint64_t *tile_sums,
                      uint64_t *total, const unsigned long long *status, int grid, cudaStream_t st) {
     int g = grid_for(cap, SCAN_TILE, grid);
-    k_scan_u64_reduce<<<g, SCAN_THREADS, 0, st>>>(a, n_dev, cap, tile_sums, status);
-    k_scan_u64_tiles<<<1, 1024, 0, st>>>(tile_sums, n_dev, cap, status);
-    k_scan_u64_apply<<<g, SCAN_THREADS, 0, st>>>(a, n_dev, cap, tile_sums, total, status);
+    launch_after(k_scan_u64_reduce, g, SCAN_THREADS, 0, st, (const uint64_t *)a, n_dev, cap,
+                 tile_sums, status);
+    launch_after(k_scan_u64_tiles, 1, 1024, 0, st, tile_sums, n_dev, cap, status);
+    launch_after(k_scan_u64_apply, g, SCAN_THREADS, 0, st, a, n_dev, cap,
+                 (const uint64_t *)tile_sums, total, status);
 }
 
 size_t scan_u64_tile_count(uint64_t cap) { return (cap + SCAN_TILE - 1) / SCAN_TILE + 1; }
@@ -633,10 +644,9 @@ void launch_combine_write(const uint32_t *road_nhit, const uint64_t *n_roads, ui
                           const uint64_t *comb_off, uint64_t comb_cap, uint32_t xft_pairs,
                           uint32_t *comb_road, uint32_t *comb_hits, unsigned long long *status,
                           int grid, cudaStream_t st) {
-    k_combine_write<false><<<grid_for(road_cap * 32, 256, grid), 256, 0, st>>>(
-        road_nhit, n_roads, road_cap, comb_off, comb_cap, xft_pairs, comb_road, comb_hits, status);
-    k_combine_write<true><<<grid_for(road_cap, 256, grid), 256, 0, st>>>(
-        road_nhit, n_roads, road_cap, comb_off, comb_cap, xft_pairs, comb_road, comb_hits, status);
+    launch_after(k_combine_write, grid_for((comb_cap + WRITE_PER - 1) / WRITE_PER, WRITE_THREADS, grid),
+                 WRITE_THREADS, 0, st, road_nhit, n_roads, road_cap, comb_off, comb_cap, xft_pairs,
+                 comb_road, comb_hits, status);
 }
 
 void launch_fit_plain(const uint32_t *words, const uint32_t *road_word, const uint32_t *road_nhit,
@@ -645,27 +655,25 @@ void launch_fit_plain(const uint32_t *words, const uint32_t *road_word, const ui
                       const int16_t *q, const svt_config cfg, uint32_t *fit_chi2,
                       int32_t *fit_par, const unsigned long long *status, int grid,
                       cudaStream_t st) {
-    k_fit_plain<<<grid_for((comb_cap + FIT_TILE - 1) / FIT_TILE * FIT_THREADS, FIT_THREADS, grid),
-                  FIT_THREADS, 0, st>>>(
-        words, road_word, road_nhit, comb_road, comb_hits, n_combs, comb_cap, F, q, cfg, fit_chi2,
-        fit_par, status);
+    launch_after(k_fit_plain,
+                 grid_for((comb_cap + FIT_TILE - 1) / FIT_TILE * FIT_THREADS, FIT_THREADS, grid),
+                 FIT_THREADS, 0, st, words, road_word, road_nhit, comb_road, comb_hits, n_combs,
+                 comb_cap, F, q, cfg, fit_chi2, fit_par, status);
 }
 
 void launch_select(const uint32_t *fit_chi2, const int32_t *fit_par, uint64_t comb_cap,
                    const uint64_t *comb_off, const uint32_t *road_flags, const uint64_t *n_roads,
                    uint64_t road_cap, const svt_config cfg, svt_best *best,
                    const unsigned long long *status, int grid, cudaStream_t st) {
-    k_select<false><<<grid_for(road_cap * 32, 256, grid), 256, 0, st>>>(
-        fit_chi2, fit_par, comb_cap, comb_off, road_flags, n_roads, road_cap, cfg, best, status);
-    k_select<true><<<grid_for(road_cap, 256, grid), 256, 0, st>>>(
-        fit_chi2, fit_par, comb_cap, comb_off, road_flags, n_roads, road_cap, cfg, best, status);
+    launch_after(k_select, grid_for(road_cap, SELECT_GROUP, grid), SELECT_THREADS, 0, st, fit_chi2,
+                 fit_par, comb_cap, comb_off, road_flags, n_roads, road_cap, cfg, best, status);
 }
 
 void launch_format(const svt_best *best, const uint32_t *words, const uint32_t *road_word,
                    const uint64_t *n_roads, uint64_t road_cap, uint32_t *out,
                    const unsigned long long *status, int grid, cudaStream_t st) {
-    k_format<<<grid_for(road_cap, 256, grid), 256, 0, st>>>(best, words, road_word, n_roads,
-                                                           road_cap, out, status);
+    launch_after(k_format, grid_for(road_cap, 256, grid), 256, 0, st, best, words, road_word, n_roads,
+                 road_cap, out, status);
 }
 
 }  // namespace svt
