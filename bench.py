@@ -955,7 +955,7 @@ def uneven_full(dev, flush, timer, steps=5, warmup=2):
            "tuned_on": f"{TILE_DRAW}-event draw, {tune_ms:.3f} ms per run",
            "l2": "flushed between steps (256 MB write)",
            "check": "status OK, evaluated combinations equal the closed form, all copies equal"}
-    ipf = recorded_profile("warp_instructions_per_fit_uneven", UNEVEN_NOTE)
+    ipf = recorded_profile("warp_instructions_per_fit_uneven_screened", UNEVEN_NOTE)
     if ipf is not None:
         ach = ipf * fits / fit_s / 1e9
         prof_sched = recorded_schedule(UNEVEN_NOTE)

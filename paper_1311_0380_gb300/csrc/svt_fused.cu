@@ -33,6 +33,9 @@
 //     at a time, writes their records one road per lane: recovering the hits
 //     of the best combination and forming its three parameters is scalar
 //     work that would otherwise hold all 32 lanes for every road.
+#include <algorithm>
+#include <cmath>
+
 #include "svt_kernels.cuh"
 
 namespace svt {
@@ -778,6 +781,733 @@ __device__ __forceinline__ bool form_record(const uint32_t *__restrict__ words,
     return pass;
 }
 
+// ---- large roads: screened in single precision ------------------------------------
+// Where a batch's roads are large (see SCREEN_MEAN), the exact 64-bit sums and
+// squares of every combination are all the work, and nearly every one of them
+// is far from the best: so every combination is SCREENED in single precision,
+// g_k = A_k(a) + B_k(b) and s = sum_k g_k^2, two rows to a packed fp32
+// instruction (about 5.5 warp instructions per 32 combinations instead of 18),
+// only the smallest s of each lane is kept, and the few combinations whose s can
+// belong to the best one are evaluated in exact 64-bit integers (the bound below
+// makes this exact, whatever the constants).
+// Screening parameters (host: make_screen).  For a combination let
+// v_k = acc_k / 2^oshift (k = 3..5, exact), so y_k = floor(v_k) lies within 1/2
+// of v_k - 1/2.  The screen forms g_k = v_k - 1/2 + e_k in single precision,
+// |e_k| <= E = 10 u M with u = 2^-24 and M = (6 2^30 + 2^(15+qshift)) / 2^oshift + 1
+// the largest magnitude of any partial sum: at most seven additions of terms
+// (six terms and q; one more when a track-trigger pair is folded), each
+// within u M, and the terms' own roundings, together within 2 u M.  Hence
+//     | |y| - |g| | <= delta = sqrt(3) (1/2 + E)      (Euclidean norms),
+// and s = fl(|g|^2) is within a factor 1 +- 2^-21 of |g|^2.  So
+//   - a combination of chi2 <= X has s <= reach(X, delta),
+//   - when some combination has s = m, the best one has
+//     s <= reach(m, 2 delta),
+// with reach(v, d) = (sqrt(v) (1 + 2^-18) + d)^2 (1 + 2^-18); the factors cover
+// every rounding of s, of the square root and of reach itself.  At the usual
+// shifts (15, 15) delta is 1.1, in units where a chi component of one
+// standard deviation is of the order of 100, so hardly any column but the
+// best one is confirmed; for extreme shifts delta grows and more columns are
+// confirmed, with the same result.
+// Clamping: a combination with |y_k| >= 32767 for some k has chi2 >= 32767^2.
+// So below SAT = 32767^2 the clamped and the unclamped chi2 order alike, the
+// screen starts at reach(min(cut, SAT), delta), and when nothing below SAT
+// turns up while the cut would let larger values pass, every combination of
+// the road (or item) is evaluated exactly (sweep).
+struct Screen {
+    float f_scale, q_scale;   // 2^-oshift, 2^(qshift - oshift)
+    float delta, thr;         // delta; reach(min(cut, SAT), delta)
+};
+constexpr uint32_t SAT = 32767u * 32767u;
+
+// A road's working set in shared memory.
+constexpr uint32_t SCREEN_ROWS = 64;
+struct ScreenSmem {
+    float4 T[N_LAYERS * MAX_HITS];   // hit i of layer l at [l*16+i]: its terms
+                                     // F[3+k][l] x 2^-oshift, k = 0..2, and in .w the bits of
+                                     // its coordinate x
+    float4 S[32];                    // suffix sums below the top suffix layer [b']
+    // rows of the chunk in pairs (a, a + 1) for the packed arithmetic, with one
+    // more pair for the last row of a road cut off by max_comb
+    float4 A34[SCREEN_ROWS / 2 + 1];   // {A_3(a), A_3(a+1), A_4(a), A_4(a+1)}, incl. q and -1/2
+    float2 A5[SCREEN_ROWS / 2 + 2];    // {A_5(a), A_5(a+1)}
+    float4 Ff[N_LAYERS];               // F[3+k][l] 2^-oshift, k = 0..2
+    int4 Fi[N_LAYERS];                 // F[3+k][l]
+    uint2 nm[N_LAYERS];                // n'_l = max(n_l, 1) and its division magic
+    uint32_t off[N_LAYERS];            // index of the first hit of layer l in the road
+    int32_t q[4];                      // q[3+k]
+};
+
+// Listed combinations whose exact chi2 is still to be formed: of every road
+// the warp has finished up to LIST_MAX, one after another (one entry with
+// combination NONE for a road without any).  When the next road's might not
+// fit (and when the warp runs out of work) they are evaluated exactly, one per
+// lane, and the roads' records written (flush_records), so that neither the
+// exact sums nor the records hold all 32 lanes for every road.
+constexpr uint32_t NONE = 0xFFFFFFFFu;
+constexpr uint32_t LIST_MAX = 8, CAND = 96;
+struct CandList {
+    uint2 ent[32];        // road, combination
+    uint2 cand[CAND];     // combinations of the road at hand that are within reach,
+                          // each with the bits of its s
+};
+
+// flush_records works where the road's tables were: per entry six record words,
+// 18 words of F (19: odd, so that the lanes' reads fall in different banks),
+// three of q
+union ScreenSlot {
+    ScreenSmem road;
+    uint32_t flush[32 * (6 + 19 + 3)];
+};
+static_assert(sizeof(ScreenSlot) <= sizeof(WarpSmem) && alignof(ScreenSlot) <= 16,
+              "a road slot holds either form");
+
+// Two packed single-precision operations at once (each half rounded to
+// nearest, as the scalar operations are).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 both(float v) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float min2(f32x2 s, float m) {   // the smaller half, and m
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(s));
+    return fminf(fminf(a, b), m);
+}
+
+// see Screen (the approximate root is within 2^-23 of the root)
+__device__ __forceinline__ float reach(float v, float d) {
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+    r = fmaf(r, 1.f + 0x1p-18f, d);
+    return r * r * (1.f + 0x1p-18f);
+}
+
+// Constants, hit coordinates and per-hit chi terms of road D in the warp's slot.
+// Global loads are issued before any shared-memory work; a road has at most 96
+// hits, so three passes of the lanes hold them all.
+__device__ __forceinline__ void screen_load(ScreenSmem &sm, const uint32_t *__restrict__ words,
+                                          const RoadDesc &D, const Geo &g,
+                                          const int16_t *__restrict__ F,
+                                          const int16_t *__restrict__ q, const Screen &sc,
+                                          uint32_t xft, const Lanes<32> &L) {
+    constexpr uint32_t MH = (uint32_t)MAX_HITS;
+    // the chi rows k = 3..5 only (18 + 3 constants): the record's parameter
+    // rows are read from global memory by the lane that forms it
+    const uint32_t rw = D.a.x, packed = D.a.y, gl = L.gl;
+    const size_t cs = (size_t)rd_sector(D.a.z) * 64 + g.mask;
+    const int32_t fv =
+        gl < 18 ? __ldg(F + cs * 36 + 18 + gl) : (gl < 21 ? __ldg(q + cs * 6 + gl - 15) : 0);
+    uint32_t hv[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const uint32_t h = gl + 32u * j;
+        hv[j] = h < g.total_hits ? __ldg(words + rw + 1 + h) : 0u;
+    }
+    const uint32_t nl = gl < N_LAYERS ? nhit_of(packed, gl) : 0u;
+    uint32_t incl = nl;   // inclusive prefix of the layer counts
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) {
+        const uint32_t v = __shfl_up_sync(L.mask, incl, d);
+        if (gl >= (uint32_t)d) incl += v;
+    }
+    if (gl < N_LAYERS) {
+        // with track-trigger pairs layer 5 is no digit of its own (radix 1)
+        const uint32_t np = (nl && !(xft && gl == N_LAYERS - 1)) ? nl : 1u;
+        sm.nm[gl] = make_uint2(np, kDivMagic[np]);
+        sm.off[gl] = incl - nl;
+        // a layer without hits contributes x = 0
+        if (nl == 0) sm.T[gl * MH] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (gl < 18) {
+        const uint32_t k = gl / 6, l = gl - 6 * k;
+        reinterpret_cast<float *>(&sm.Ff[l])[k] = (float)fv * sc.f_scale;
+        reinterpret_cast<int32_t *>(&sm.Fi[l])[k] = fv;
+    } else if (gl < 21) {
+        sm.q[gl - 18] = fv;
+    }
+    __syncwarp(L.mask);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const uint32_t h = gl + 32u * j;
+        if (h < g.total_hits) {
+            const uint32_t l = hit_layer(hv[j]);
+            const uint32_t i = h - sm.off[l];   // hits are sorted by layer (validated)
+            const uint32_t xc = hit_coord(hv[j]);
+            const float x = (float)xc;
+            const float4 f = sm.Ff[l];
+            sm.T[l * MH + i] = make_float4(f.x * x, f.y * x, f.z * x, __uint_as_float(xc));
+        }
+    }
+    __syncwarp(L.mask);
+    if (xft) {
+        // pair i: layer 4's entry i carries both coordinates' terms of
+        // track-trigger track i (equal counts are validated); layer 5 then
+        // adds none (its coordinates stay)
+        const uint32_t n4 = nhit_of(packed, 4);
+        for (uint32_t i = gl; i < n4; i += 32u) {
+            float4 &t4 = sm.T[4 * MH + i], &t5 = sm.T[5 * MH + i];
+            const float4 v = t5;
+            t4.x += v.x;
+            t4.y += v.y;
+            t4.z += v.z;
+            t5.x = t5.y = t5.z = 0.f;
+        }
+        __syncwarp(L.mask);
+    }
+}
+
+// S[b'] = sum over the suffix layers below the top one, b' < NBp (< 32).
+__device__ __forceinline__ void screen_suffix(ScreenSmem &sm, const Geo &g, const Lanes<32> &L) {
+    constexpr uint32_t MH = (uint32_t)MAX_HITS;
+    for (uint32_t bp = L.gl; bp < g.NBp; bp += 32u) {
+        uint32_t rem = bp;
+        float s3 = 0.f, s4 = 0.f, s5 = 0.f;
+#pragma unroll
+        for (int l = N_LAYERS - 1; l >= 1; --l) {
+            if ((uint32_t)l > g.split) {
+                const uint2 nm = sm.nm[l];
+                const uint32_t qd = div_by(rem, nm.x, nm.y);
+                const float4 t = sm.T[l * MH + rem - qd * nm.x];
+                rem = qd;
+                s3 += t.x;
+                s4 += t.y;
+                s5 += t.z;
+            }
+        }
+        sm.S[bp] = make_float4(s3, s4, s5, 0.f);
+    }
+}
+
+// The sums of row a (q and the -1/2 of the screen included) at index `slot`
+// of the chunk's rows.
+__device__ __forceinline__ void screen_row(ScreenSmem &sm, uint32_t split, uint32_t a, uint32_t slot,
+                                          const Screen &sc) {
+    constexpr uint32_t MH = (uint32_t)MAX_HITS;
+    uint32_t rem = a;
+    float a3 = fmaf((float)sm.q[0], sc.q_scale, -0.5f);
+    float a4 = fmaf((float)sm.q[1], sc.q_scale, -0.5f);
+    float a5 = fmaf((float)sm.q[2], sc.q_scale, -0.5f);
+#pragma unroll
+    for (int l = N_LAYERS - 2; l >= 0; --l) {
+        if ((uint32_t)l < split) {
+            const uint2 nm = sm.nm[l];
+            const uint32_t qd = div_by(rem, nm.x, nm.y);
+            const float4 t = sm.T[l * MH + rem - qd * nm.x];
+            rem = qd;
+            a3 += t.x;
+            a4 += t.y;
+            a5 += t.z;
+        }
+    }
+    float *p34 = reinterpret_cast<float *>(sm.A34 + slot / 2) + (slot & 1u);
+    p34[0] = a3;
+    p34[2] = a4;
+    reinterpret_cast<float *>(sm.A5)[slot] = a5;
+}
+
+// chi2 of combination c exactly: the sums in int64 (Eq. 1), the floor, the
+// clamp and the squares.
+__device__ __forceinline__ uint32_t exact_chi2(const ScreenSmem &sm, uint32_t c, const svt_config &cfg) {
+    constexpr uint32_t MH = (uint32_t)MAX_HITS;
+    long long acc[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        acc[k] = (long long)((unsigned long long)(long long)sm.q[k] << cfg.qshift);
+    uint32_t digit[N_LAYERS], rem = c;
+#pragma unroll
+    for (int l = N_LAYERS - 1; l >= 0; --l) {
+        const uint2 nm = sm.nm[l];
+        const uint32_t qd = div_by(rem, nm.x, nm.y);
+        digit[l] = rem - qd * nm.x;
+        rem = qd;
+    }
+    if (cfg.xft_pairs) digit[N_LAYERS - 1] = digit[N_LAYERS - 2];   // the pair's own index
+#pragma unroll
+    for (int l = 0; l < N_LAYERS; ++l) {
+        const int32_t x = (int32_t)__float_as_uint(sm.T[l * MH + digit[l]].w);
+        const int4 f = sm.Fi[l];
+        acc[0] += (long long)f.x * x;
+        acc[1] += (long long)f.y * x;
+        acc[2] += (long long)f.z * x;
+    }
+    uint32_t chi2 = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int32_t y = clamp_chi((int32_t)(acc[k] >> cfg.oshift));   // |y| < 2^31
+        chi2 += (uint32_t)(y * y);
+    }
+    return chi2;
+}
+
+// Best key over the combinations [c_lo, c_hi), every one evaluated exactly;
+// key = (chi2 << 32) | c, UINT64_MAX when none passes the cut.
+__device__ __forceinline__ unsigned long long sweep(const ScreenSmem &sm, uint32_t c_lo, uint32_t c_hi,
+                                                    const svt_config &cfg, const Lanes<32> &L) {
+    unsigned long long best = ~0ull;
+    for (uint32_t c = c_lo + L.gl; c < c_hi; c += 32u) {
+        const uint32_t chi2 = exact_chi2(sm, c, cfg);
+        const unsigned long long key = ((unsigned long long)chi2 << 32) | c;
+        if (chi2 <= cfg.chi2_cut && key < best) best = key;
+    }
+    return group_min64<32>(best, L);
+}
+
+// The combinations of rows [a_lo, a_hi) that can be the best one, by a whole
+// warp: listed in cand, their number returned (more than CAND: they did not
+// fit); thr is the final reach.  Each lane takes one column and runs down the
+// rows of the chunk, two per step; in the last pass over the columns, when only
+// w < 32 of them are left, the lanes form floor(32 / w) groups of w and each
+// group takes one block of the row pairs.  A lane keeps its smallest s, the pass
+// it is from and the smallest of its other passes; at the end of the chunk the
+// columns that hold combinations within reach are looked at once more, a row
+// per lane.
+__device__ __forceinline__ uint32_t list_rows(ScreenSmem &sm, uint2 *cand, const Geo &g, uint32_t a_lo,
+                                              uint32_t a_hi, const Screen &sc, float &thr,
+                                              uint32_t lane) {
+    constexpr uint32_t MH = (uint32_t)MAX_HITS, NR = SCREEN_ROWS, ALL = 0xffffffffu;
+    constexpr float FAR = 1e18f;   // a row past the last: its s is never the smallest
+    uint32_t listed = 0;
+    thr = sc.thr;
+    const uint32_t NB = g.NB, NA = g.NA, C_eval = g.C_eval, NBp = g.NBp, top = g.split;
+    const uint32_t mp = kDivMagic[NBp], n_passes = (NB + 31u) >> 5;
+    for (uint32_t ac = a_lo; ac < a_hi; ac += NR) {
+        const uint32_t ae = min(ac + NR, a_hi);
+        // the road's last row when max_comb cuts it short: kept apart, in the
+        // extra pair, for the columns that are left of it
+        const bool cut_row = ae == NA && NA * NB > C_eval;
+        const uint32_t rows = ae - ac - (cut_row ? 1u : 0u), pairs = (rows + 1u) >> 1;
+#pragma unroll
+        for (uint32_t r0 = 0; r0 < NR; r0 += 32u) {
+            const uint32_t r = r0 + lane;
+            if (r < ae - ac) screen_row(sm, top, ac + r, r < rows ? r : NR, sc);
+        }
+        if (lane == 0 && (rows & 1u)) {
+            reinterpret_cast<float *>(sm.A34 + rows / 2)[1] = FAR;
+            reinterpret_cast<float *>(sm.A34 + rows / 2)[3] = 0.f;
+            reinterpret_cast<float *>(sm.A5)[rows] = 0.f;
+        }
+        __syncwarp();
+        auto screen = [&](uint32_t p, f32x2 b3, f32x2 b4, f32x2 b5) {
+            const ulonglong2 v = reinterpret_cast<const ulonglong2 *>(sm.A34)[p];
+            const f32x2 g3 = add2(v.x, b3), g4 = add2(v.y, b4),
+                        g5 = add2(reinterpret_cast<const f32x2 *>(sm.A5)[p], b5);
+            return fma2(g5, g5, fma2(g4, g4, mul2(g3, g3)));
+        };
+        // lane `ln`'s column in pass cp and its row pairs
+        struct Column {
+            uint32_t b, lo, hi;
+            bool extra;
+        };
+        auto column = [&](uint32_t cp, uint32_t ln) {
+            Column c{cp * 32u + ln, 0u, pairs, cut_row};
+            const uint32_t w = NB - cp * 32u;
+            if (w < 32u) {   // uniform: the last, partial pass
+                const uint32_t mw = kDivMagic[w];
+                const uint32_t grp = div_by(ln, w, mw), n_grp = div_by(32u, w, mw);
+                const uint32_t len = div_by(pairs + n_grp - 1u, n_grp, kDivMagic[n_grp]);
+                c.b -= grp * w;
+                c.lo = min(grp * len, pairs);   // groups past the last pair get none
+                c.hi = min(c.lo + len, pairs);
+                c.extra = cut_row && grp == 0;
+            }
+            c.extra = c.extra && (NA - 1u) * NB + c.b < C_eval;
+            return c;
+        };
+        // column b = is * NBp + bp: hit `is` of the top suffix layer and entry bp
+        // of the suffix table
+        auto column_sums = [&](uint32_t b) {
+            const uint32_t is = div_by(b, NBp, mp), bp = b - is * NBp;
+            const float4 t = sm.T[top * MH + is], u = sm.S[bp];
+            return make_float3(t.x + u.x, t.y + u.y, t.z + u.z);
+        };
+        auto smallest = [&](const Column &c) {
+            const float3 B = column_sums(c.b);
+            const f32x2 b3 = both(B.x), b4 = both(B.y), b5 = both(B.z);
+            float m = 3e38f;
+#pragma unroll 4
+            for (uint32_t p = c.lo; p < c.hi; ++p) m = min2(screen(p, b3, b4, b5), m);
+            if (cut_row && c.extra)
+                m = fminf(__uint_as_float((uint32_t)screen(NR / 2, b3, b4, b5)), m);
+            return m;
+        };
+        float m1 = 3e38f, m2 = 3e38f;
+        uint32_t cp1 = 0;
+        for (uint32_t cp = 0; cp < n_passes; ++cp) {
+            const float m = smallest(column(cp, lane));
+            m2 = fminf(m2, fmaxf(m, m1));
+            cp1 = m < m1 ? cp : cp1;
+            m1 = fminf(m, m1);
+        }
+        // the smallest s so far (s >= 0: its bits order like it)
+        const float ms = __uint_as_float(__reduce_min_sync(ALL, __float_as_uint(m1)));
+        if (ms <= thr) {   // uniform
+            thr = fminf(thr, reach(ms, 2.f * sc.delta));
+            // the lanes with something within reach, for the pass their smallest s is
+            // from; when one has more in another pass, every pass again
+            const bool again = __any_sync(ALL, m2 <= thr);
+            for (uint32_t cp = 0; cp < (again ? n_passes : 1u); ++cp) {
+                const float m = again ? smallest(column(cp, lane)) : m1;
+                uint32_t todo = __ballot_sync(ALL, m <= thr);
+                while (todo) {
+                    const uint32_t src = (uint32_t)__ffs(todo) - 1u;
+                    todo &= todo - 1u;
+                    const Column c = column(again ? cp : __shfl_sync(ALL, cp1, src), src);
+                    const float3 B = column_sums(c.b);
+                    const uint32_t r_lo = 2u * c.lo, r_hi = min(2u * c.hi, rows);
+                    const uint32_t n_r = r_hi > r_lo ? r_hi - r_lo : 0u;
+                    const uint32_t n_x = n_r + (c.extra ? 1u : 0u);
+                    for (uint32_t i0 = 0; i0 < n_x; i0 += 32u) {
+                        const uint32_t i = i0 + lane, sl = i < n_r ? r_lo + i : NR;   // row slot
+                        const float *p =
+                            reinterpret_cast<const float *>(sm.A34 + sl / 2) + (sl & 1u);
+                        const float g3 = __fadd_rn(p[0], B.x), g4 = __fadd_rn(p[2], B.y),
+                                    g5 = __fadd_rn(reinterpret_cast<const float *>(sm.A5)[sl], B.z);
+                        const float s = __fmaf_rn(g5, g5, __fmaf_rn(g4, g4, __fmul_rn(g3, g3)));
+                        const bool hit = i < n_x && s <= thr;
+                        const uint32_t hits = __ballot_sync(ALL, hit);
+                        const uint32_t k = listed + __popc(hits & ((1u << lane) - 1u));
+                        if (hit && k < CAND)
+                            cand[k] = make_uint2((i < n_r ? ac + r_lo + i : NA - 1u) * NB + c.b,
+                                                 __float_as_uint(s));
+                        listed += __popc(hits);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        // what later columns and rows have put out of reach leaves the list
+        if (listed > 1u && listed <= CAND) {   // uniform
+            uint32_t kept = 0;
+            for (uint32_t k0 = 0; k0 < listed; k0 += 32u) {
+                const uint2 e = k0 + lane < listed ? cand[k0 + lane] : make_uint2(0u, ~0u);
+                const bool keep = k0 + lane < listed && __uint_as_float(e.y) <= thr;
+                const uint32_t kb = __ballot_sync(ALL, keep);
+                if (keep) cand[kept + __popc(kb & ((1u << lane) - 1u))] = e;
+                kept += __popc(kb);
+                __syncwarp();
+            }
+            listed = kept;
+        }
+    }
+    return listed;
+}
+
+// Best key of rows [a_lo, a_hi) by a whole warp: the listed combinations, or all
+// of them where they did not fit the list or nothing is sure to lie below SAT
+// (see Screen), evaluated exactly.
+__device__ __forceinline__ unsigned long long best_of_list(const ScreenSmem &sm, const uint2 *cand,
+                                                           uint32_t listed, float thr,
+                                                           uint32_t c_lo, uint32_t c_hi,
+                                                           const svt_config &cfg,
+                                                           const Lanes<32> &L) {
+    if (listed > CAND || (cfg.chi2_cut >= SAT && !(thr < (float)SAT)))
+        return sweep(sm, c_lo, c_hi, cfg, L);
+    unsigned long long best = ~0ull;
+    for (uint32_t k = L.gl; k < listed; k += 32u) {
+        const uint32_t c = cand[k].x, chi2 = exact_chi2(sm, c, cfg);
+        const unsigned long long key = ((unsigned long long)chi2 << 32) | c;
+        if (chi2 <= cfg.chi2_cut && key < best) best = key;
+    }
+    return group_min64<32>(best, L);
+}
+
+// A road of at most DIRECT passes of a group's lanes over its combinations is
+// evaluated exactly at once, without the tables.
+constexpr uint32_t DIRECT = 2;
+
+// One road fitted whole by the warp: its candidates in cand, their number
+// returned (at most LIST_MAX).
+__device__ __forceinline__ uint32_t screen_road(ScreenSmem &sm, uint2 *cand,
+                                              const uint32_t *__restrict__ words,
+                                              const RoadDesc &D, const int16_t *__restrict__ F,
+                                              const int16_t *__restrict__ q,
+                                              const svt_config &cfg, const Screen &sc,
+                                              const Lanes<32> &L) {
+    const Geo g = geo_of(D);
+    if (g.C_eval == 0) return 0;
+    screen_load(sm, words, D, g, F, q, sc, cfg.xft_pairs, L);
+    unsigned long long best;
+    if (g.C_eval <= DIRECT * 32u) {
+        best = sweep(sm, 0, g.C_eval, cfg, L);
+    } else {
+        screen_suffix(sm, g, L);
+        float thr;
+        const uint32_t n = list_rows(sm, cand, g, 0, g.NA, sc, thr, L.gl);
+        if (n <= LIST_MAX && (cfg.chi2_cut < SAT || thr < (float)SAT)) return n;
+        best = best_of_list(sm, cand, n, thr, 0, g.C_eval, cfg, L);
+    }
+    __syncwarp();
+    if (L.gl == 0) cand[0].x = (uint32_t)best;   // (UINT64_MAX reads as NONE)
+    return 1;
+}
+
+// The coordinates of combination c's hits in the road with descriptor words da
+// (svt_roads.cuh), by one lane: the hits are the digits of c in the radices
+// n'_l.  Every load is issued before any is used (a layer without hits reads
+// the road's header word and discards it: x = 0).
+__device__ __forceinline__ void comb_coords(const uint32_t *__restrict__ words,
+                                            const svt_config &cfg, const uint4 &da, uint32_t c,
+                                            int32_t (&x)[N_LAYERS]) {
+    const uint32_t packed = da.y;
+    uint32_t digit[N_LAYERS], rem = c;
+#pragma unroll
+    for (int l = N_LAYERS - 1; l >= 0; --l) {
+        const uint32_t nl = nhit_of(packed, l);
+        const uint32_t np = (nl && !(cfg.xft_pairs && l == N_LAYERS - 1)) ? nl : 1u;
+        const uint32_t qd = div_by(rem, np, kDivMagic[np]);
+        digit[l] = rem - qd * np;
+        rem = qd;
+    }
+    if (cfg.xft_pairs) digit[N_LAYERS - 1] = digit[N_LAYERS - 2];   // the pair's own index
+    uint32_t hw[N_LAYERS];
+    uint32_t off = da.x + 1;   // first hit word of layer l (hits are sorted by layer)
+#pragma unroll
+    for (int l = 0; l < N_LAYERS; ++l) {
+        const uint32_t nl = nhit_of(packed, l);
+        hw[l] = __ldg(words + (nl ? off + digit[l] : da.x));
+        off += nl;
+    }
+#pragma unroll
+    for (int l = 0; l < N_LAYERS; ++l) x[l] = nhit_of(packed, l) ? (int32_t)hit_coord(hw[l]) : 0;
+}
+
+// y_k = floor((q_k 2^qshift + sum_l F_kl x_l) / 2^oshift) (Eq. 1), in int64
+template <typename GetF>
+__device__ __forceinline__ int32_t exact_y(const svt_config &cfg, int32_t qk, GetF F,
+                                           const int32_t (&x)[N_LAYERS]) {
+    long long acc = (long long)qk * (1ll << cfg.qshift);
+#pragma unroll
+    for (int l = 0; l < N_LAYERS; ++l) acc += (long long)F(l) * (long long)x[l];
+    return (int32_t)(acc >> cfg.oshift);   // |y| < 2^31
+}
+
+__device__ __forceinline__ uint32_t chi_square(int32_t y3, int32_t y4, int32_t y5) {
+    const int32_t a = clamp_chi(y3), b = clamp_chi(y4), c = clamp_chi(y5);
+    return (uint32_t)(a * a) + (uint32_t)(b * b) + (uint32_t)(c * c);
+}
+
+// Records of the n_rec listed combinations: each lane forms one, the first
+// lane of every road picks the road's best one, and the warp stores the records
+// with consecutive lanes on consecutive words.  The entries' rows of constants
+// (84 bytes each, scattered over the table) are fetched by the whole warp, word
+// after word, and read back by the entry's lane: lane by lane every one of 42
+// loads touched 32 cache lines, 18 us of the paper's shape at 3000 events.
+// Returns the passing roads this lane picked for.
+__device__ __forceinline__ uint32_t flush_records(const uint32_t *__restrict__ words,
+                                                  const RoadDesc *__restrict__ desc,
+                                                  const int16_t *__restrict__ F,
+                                                  const int16_t *__restrict__ q,
+                                                  const svt_config &cfg, uint32_t *out,
+                                                  CandList &rl, uint32_t *stage,
+                                                  uint32_t n_rec) {
+    const uint32_t lane = threadIdx.x & 31u;
+    __syncwarp();
+    uint32_t *Fs = stage + 32 * 6, *qs = Fs + 32 * 19;
+    const uint2 e = rl.ent[lane];
+    const bool on = lane < n_rec;
+    const bool head = on && (lane == 0 || rl.ent[lane - 1].x != e.x);
+    uint4 da = make_uint4(0, 0, 0, 0);
+    uint32_t geo = 0;
+    if (on) {
+        da = __ldg(&desc[e.x].a);
+        geo = __ldg(&desc[e.x].b.x);
+    }
+    const uint32_t cs = rd_sector(da.z) * 64u + ((geo >> 13) & 63u);
+    if ((((uintptr_t)F | (uintptr_t)q) & 3u) == 0) {
+        const uint32_t *F32 = reinterpret_cast<const uint32_t *>(F);
+        const uint32_t *q32 = reinterpret_cast<const uint32_t *>(q);
+#pragma unroll 4
+        for (uint32_t j = 0; j * 32u < n_rec * 21u; ++j) {
+            const uint32_t i = j * 32u + lane, k = i / 21u, w = i - k * 21u;
+            const uint32_t c = __shfl_sync(0xffffffffu, cs, k);
+            if (k < n_rec) {
+                if (w < 18u)
+                    Fs[k * 19u + w] = __ldg(F32 + c * 18u + w);
+                else
+                    qs[k * 3u + w - 18u] = __ldg(q32 + c * 3u + w - 18u);
+            }
+        }
+    } else {
+        uint16_t *Fh = reinterpret_cast<uint16_t *>(Fs), *qh = reinterpret_cast<uint16_t *>(qs);
+        for (uint32_t j = 0; j * 32u < n_rec * 42u; ++j) {
+            const uint32_t i = j * 32u + lane, k = i / 42u, w = i - k * 42u;
+            const uint32_t c = __shfl_sync(0xffffffffu, cs, k);
+            if (k < n_rec) {
+                if (w < 36u)
+                    Fh[k * 38u + w] = (uint16_t)__ldg(F + c * 36u + w);
+                else
+                    qh[k * 6u + w - 36u] = (uint16_t)__ldg(q + c * 6u + w - 36u);
+            }
+        }
+    }
+    int32_t x[N_LAYERS] = {0, 0, 0, 0, 0, 0};
+    if (on && e.y != NONE) comb_coords(words, cfg, da, e.y, x);
+    __syncwarp();
+    uint32_t *mine = stage + lane * 6;
+    if (on) {
+        // 16-bit entry i of a row of pairs (little-endian: even ones in the low half)
+        auto at16 = [](const uint32_t *w, int i) {
+            return (i & 1) ? (int32_t)w[i >> 1] >> 16 : (int32_t)(int16_t)(w[i >> 1] & 0xFFFFu);
+        };
+        int32_t y[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            y[k] = exact_y(cfg, at16(qs + lane * 3, k),
+                           [&](int l) { return at16(Fs + lane * 19, k * 6 + l); }, x);
+        const uint32_t chi2 = chi_square(y[3], y[4], y[5]);
+        const bool pass = e.y != NONE && chi2 <= cfg.chi2_cut;
+        uint32_t flags = pass ? SVT_FLAG_PASS : 0u;
+        if (((geo >> 19) & 127u) == 0) flags |= SVT_FLAG_NO_HITS;
+        if (geo & (1u << 27)) flags |= SVT_FLAG_BAD_PATTERN;
+        if (geo & (1u << 26)) flags |= SVT_FLAG_OVERFLOW;
+        mine[0] = rd_id(da.z) | (flags << 24);
+        mine[1] = pass ? e.y : NONE;
+        mine[2] = pass ? chi2 : 0u;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) mine[3 + k] = pass ? (uint32_t)y[k] : 0u;
+    }
+    __syncwarp();
+    uint32_t pick = lane, n_pass = 0;
+    if (head) {
+        bool ok = mine[1] != NONE;
+        for (uint32_t t = lane + 1; t < n_rec && rl.ent[t].x == e.x; ++t) {
+            const uint32_t *a = stage + t * 6, *b = stage + pick * 6;
+            if (a[1] != NONE && (!ok || a[2] < b[2] || (a[2] == b[2] && a[1] < b[1]))) {
+                pick = t;
+                ok = true;
+            }
+        }
+        n_pass = ok ? 1u : 0u;
+    }
+    const uint32_t heads = __ballot_sync(0xffffffffu, head), n_out = __popc(heads) * 6u;
+    if (head) rl.ent[__popc(heads & ((1u << lane) - 1u))] = make_uint2(e.x, pick);
+    __syncwarp();
+    for (uint32_t i = lane; i < n_out; i += 32) {
+        const uint32_t k = i / 6;
+        const uint2 o = rl.ent[k];
+        out[(size_t)o.x * 6 + (i - k * 6)] = stage[o.y * 6 + (i - k * 6)];
+    }
+    __syncwarp();
+    return n_pass;
+}
+
+// The fit of a whole batch by screening: items of split roads, then chunks of
+// consecutive roads, each road by one warp.  Returns the passing roads whose
+// records this lane wrote.
+__device__ __forceinline__ uint32_t screen_path(
+    ScreenSlot &slot, CandList &rl, const uint32_t *__restrict__ words,
+    const RoadDesc *__restrict__ desc, const int16_t *__restrict__ F,
+    const int16_t *__restrict__ q, const svt_config &cfg, const Screen &sc, const FusedRoads &fr,
+    uint32_t n_big, uint32_t n_items, uint32_t R, uint32_t roads_per_chunk, uint32_t *out) {
+    ScreenSmem &sm = slot.road;
+    const BigList &bl = fr.bl;
+    const int lane = threadIdx.x & 31;
+    const Lanes<32> LW = lanes_of<32>(lane);
+    uint32_t n_rec = 0, n_pass = 0;   // entries of rl (uniform over the warp)
+    auto flush = [&]() {
+        n_pass += flush_records(words, desc, F, q, cfg, out, rl, slot.flush, n_rec);
+        n_rec = 0;
+    };
+    for (;;) {
+        uint32_t it = 0;
+        if (lane == 0) it = atomicAdd(bl.counters + 0, 1u);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= n_items) break;
+        const uint32_t j = find_slot(bl.item_off, n_big, it, lane);
+        const uint32_t r = __ldg(bl.road + j);
+        const uint32_t k = it - __ldg(bl.item_off + j);
+        RoadDesc D;
+        D.a = __ldg(&desc[r].a);
+        D.b = __ldg(&desc[r].b);
+        const Geo g = geo_of(D);
+        screen_load(sm, words, D, g, F, q, sc, cfg.xft_pairs, LW);
+        screen_suffix(sm, g, LW);
+        const uint32_t a_lo = k * fr.rows;
+        const uint32_t a_hi = min(a_lo + fr.rows, g.NA);
+        float thr;
+        const uint32_t n_c = list_rows(sm, rl.cand, g, a_lo, a_hi, sc, thr, (uint32_t)lane);
+        const unsigned long long best = best_of_list(sm, rl.cand, n_c, thr, a_lo * g.NB,
+                                                     min(a_hi * g.NB, g.C_eval), cfg, LW);
+        uint32_t last = 0;
+        if (lane == 0) {
+            if (best != ~0ull) atomicMin(fr.key + r, best);
+            __threadfence();
+            last = (atomicSub(bl.pending + j, 1u) == 1u) ? 1u : 0u;
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+        if (last) {   // every item of road r is done: list it with its final key
+            if (n_rec == 32) flush();
+            if (lane == 0) {
+                __threadfence();
+                // (the low word of these keys is the combination index itself)
+                rl.ent[n_rec] = make_uint2(r, (uint32_t)__ldcg(fr.key + r));   // (or NONE)
+            }
+            n_rec += 1;
+        }
+        __syncwarp();
+    }
+    for (;;) {
+        uint32_t k = 0;
+        if (lane == 0) k = atomicAdd(bl.counters + 1, 1u);
+        k = __shfl_sync(0xffffffffu, k, 0);
+        if ((uint64_t)k * roads_per_chunk >= R) break;
+        const uint32_t c0 = k * roads_per_chunk;
+        const uint32_t n = min(roads_per_chunk, R - c0);
+        uint4 da = make_uint4(0, 0, 0, 0), db = make_uint4(0, 0, 0, 0);
+        if ((uint32_t)lane < n) {
+            da = __ldg(&desc[c0 + lane].a);
+            db = __ldg(&desc[c0 + lane].b);
+        }
+        for (uint32_t jj = 0; jj < n; ++jj) {
+            const RoadDesc D = shfl_desc(da, db, jj);
+            if (D.a.w > fr.small_max) continue;   // split road: done above
+            if (n_rec > 32u - LIST_MAX) flush();
+            const uint32_t n_c = screen_road(sm, rl.cand, words, D, F, q, cfg, sc, LW);
+            __syncwarp();
+            const uint32_t n_e = max(n_c, 1u);   // at most LIST_MAX
+            if ((uint32_t)lane < n_e)
+                rl.ent[n_rec + lane] = make_uint2(c0 + jj, n_c ? rl.cand[lane].x : NONE);
+            n_rec += n_e;
+            __syncwarp();
+        }
+    }
+    if (n_rec) flush();
+    return n_pass;
+}
+
+constexpr size_t LIST_BYTES =
+    sizeof(RecordList) > sizeof(CandList) ? sizeof(RecordList) : sizeof(CandList);
+static_assert(LIST_BYTES % 16 == 0, "lists keep 16-byte alignment");
+// Mean evaluated combinations of a batch's roads from which on the batch is
+// fitted by screening (one road per warp, GROUP 1; one form per launch, so that
+// the warps keep to one path of code).  Its set-up, listing and exact step cost
+// about 250 warp instructions a road more than the exact form's, its loop 13 less
+// per 32 combinations: fit kernel, exact / screened, in us, 1500 events of 64
+// roads: mean 244 combinations 80 / 92, 582: 119 / 123, 731: 121 / 121, 994: 143 /
+// 142, 1337: 201 / 199, 1837: 207 / 178, 2927 (256-row items): 267 / 190, 3981: 338
+// / 227, 4096: 287 / 190; at 100 events the line lies at the same place.
+// (Screening every batch, with tables for several small roads at once, a lane
+// to a small road or size classes of 4 to 32 lanes a road, took fewer
+// instructions at small means but kept fewer warps busy: 1.1 to 1.7 times the
+// exact form's time on the scaled workload.)
+constexpr uint64_t SCREEN_MEAN = 1024;
+
 // K4: persistent fit / cut / select / format.  GROUP 2: two consecutive SMALL
 // roads of one chunk with the same geometry go to the two halves of the warp;
 // GROUP 4: four consecutive TINY roads of the same geometry go to its four
@@ -797,12 +1527,12 @@ __global__ void __launch_bounds__(GROUP == 32 ? 384 : 512, 2)
                      const Dims *__restrict__ dims, const uint32_t *__restrict__ event_road,
                      const RoadDesc *__restrict__ desc, uint64_t *counts, uint64_t road_cap,
                      const int16_t *__restrict__ F, const int16_t *__restrict__ q,
-                     const svt_config cfg, const FusedRoads fr, uint32_t roads_per_chunk,
-                     uint32_t *out, unsigned long long *status) {
+                     const svt_config cfg, const Screen sc, const FusedRoads fr,
+                     uint32_t roads_per_chunk, uint32_t *out, unsigned long long *status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     WarpSmem &sm = *reinterpret_cast<WarpSmem *>(smem_raw + SLOT_BYTES * (threadIdx.x >> 5));
-    RecordList &rl = reinterpret_cast<RecordList *>(
-        smem_raw + SLOT_BYTES * (blockDim.x >> 5))[threadIdx.x >> 5];
+    unsigned char *list = smem_raw + SLOT_BYTES * (blockDim.x >> 5) + LIST_BYTES * (threadIdx.x >> 5);
+    RecordList &rl = *reinterpret_cast<RecordList *>(list);
     const int lane = threadIdx.x & 31;
     const Lanes<32> LW = lanes_of<32>(lane);
     wait_prior_grid();   // road extraction has completed (see launch_after)
@@ -819,6 +1549,17 @@ __global__ void __launch_bounds__(GROUP == 32 ? 384 : 512, 2)
     const uint64_t R64 = counts[0];
     if (R64 > road_cap || R64 == 0) return;
     const uint32_t R = (uint32_t)R64;
+    if constexpr (GROUP == 1) {
+        if (counts[2] >= SCREEN_MEAN * R64) {
+            const uint32_t n_pass = __reduce_add_sync(
+                0xffffffffu,
+                screen_path(reinterpret_cast<ScreenSlot &>(sm), *reinterpret_cast<CandList *>(list),
+                            words, desc, F, q, cfg, sc, fr, n_big, n_items, R, roads_per_chunk, out));
+            if (lane == 0 && n_pass)
+                atomicAdd((unsigned long long *)(counts + 3), (unsigned long long)n_pass);
+            return;
+        }
+    }
     const uint32_t sh = 32u - cfg.oshift, qsh = cfg.qshift + sh;
     const uint32_t init_chi = cfg.chi2_cut == 0xFFFFFFFFu ? 0xFFFFFFFFu : cfg.chi2_cut + 1u;
     // GROUP 32: lanes to a tiny road, so that chunks of 32, 16 or at most 8
@@ -1042,8 +1783,27 @@ __global__ void __launch_bounds__(GROUP == 32 ? 384 : 512, 2)
 }  // namespace
 
 size_t fit_smem_bytes(int warps_per_block) {
-    return (SLOT_BYTES + sizeof(RecordList)) * (size_t)warps_per_block;
+    return (SLOT_BYTES + LIST_BYTES) * (size_t)warps_per_block;
 }
+
+namespace {
+
+// see Screen: rounded up at every step
+Screen make_screen(const svt_config &cfg) {
+    const double u = 0x1p-24, P = std::ldexp(1.0, -(int)cfg.oshift);
+    const double M = (6.0 * 0x1p30 + std::ldexp(1.0, 15 + (int)cfg.qshift)) * P + 1.0;
+    const double delta = std::sqrt(3.0) * (0.5 + 10.0 * u * M) * (1.0 + 1e-6);
+    const double cut = std::sqrt((double)std::min(cfg.chi2_cut, SAT)) + delta;
+    Screen sc;
+    sc.f_scale = (float)P;
+    sc.q_scale = (float)std::ldexp(1.0, (int)cfg.qshift - (int)cfg.oshift);
+    sc.delta = (float)(delta * (1.0 + 1e-6));
+    sc.thr = (float)(cut * cut * (1.0 + 1e-5));
+    return sc;
+}
+
+}  // namespace
+
 
 int fit_persistent_blocks_per_sm(int warps_per_block, uint32_t group) {
     const size_t smem = fit_smem_bytes(warps_per_block);
@@ -1081,10 +1841,11 @@ cudaError_t launch_fit_persistent(const uint32_t *words, const uint64_t *event_o
                                   uint32_t *out, unsigned long long *status,
                                   int warps_per_block, int grid, cudaStream_t st) {
     const size_t smem = fit_smem_bytes(warps_per_block);
-    const bool guarded = cfg.chi2_cut < 32767u * 32767u;
+    const bool guarded = cfg.chi2_cut < SAT;
+    const Screen sc = make_screen(cfg);
     auto launch = [&](auto kernel) {
         launch_after(kernel, grid, warps_per_block * 32, smem, st, words, event_off, dims,
-                     event_road, desc, counts, road_cap, F, q, cfg, fr, roads_per_chunk, out,
+                     event_road, desc, counts, road_cap, F, q, cfg, sc, fr, roads_per_chunk, out,
                      status);
     };
     if (guarded) {
