@@ -860,8 +860,8 @@ int svt_calib_backward(const float *d_x, const float *d_grad_y, uint64_t n_track
     if (workspace_bytes < w.bytes) return SVT_ERR_BAD_ARG;
     CalibIndex x = carve_calib_index(d_index, n_tracks, n_sectors);
     launch_calib_grad(d_x, d_grad_y, x.item_sector, x.item_start, x.sector_off, x.sector_item,
-                      x.n_items, x.max_items, n_sectors, d_F, w.item_grad, d_dF, d_dq, d_dx,
-                      tile_grid(), (cudaStream_t)stream);
+                      x.n_items, x.max_items, n_sectors, n_tracks, d_F, w.item_grad, d_dF, d_dq,
+                      d_dx, current_sm_count(), tile_grid(), (cudaStream_t)stream);
     return launch_status();
 }
 

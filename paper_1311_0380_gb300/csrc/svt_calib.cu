@@ -1096,34 +1096,218 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
     }
 }
 
+// The general backward (sum_t g_t x_t^T and sum_t g_t, g = grad_y) over tracks
+// staged by the bulk-copy unit, for x and grad_y that start on a 16-byte
+// boundary and no dx (the launcher takes k_grad_items otherwise): the runs,
+// copies and segments of k_loss_grad_bulk, 48 bytes a track, and k_lg_final for
+// the sectors' sums.  Bound by HBM: six warps of two buffers per SM (150 KB,
+// up to 23 MB in flight on the chip) read 16 M tracks in 114 us, the rate of a
+// plain copy (eight warps 117, four 119; fewer warps are fewer runs to add up).
+// A lane sums its (at most eight) tracks of an item apart and adds them to the
+// run's sums once an item: two short sums instead of one long one, and a
+// partial for every run instead of every item.  16 M tracks in 512 sectors, this
+// kernel and the final sums: 118 us, k_grad_items and k_grad_final 155; 1 M
+// tracks 17.7 and 19.0, 30 K 9.4 and 9.7 (16 sectors: 22.3 and 34.7, 9.5 and
+// 10.2); error of dF against exact sums, relative to its norm, 1.7e-7 (16 M)
+// and 1.0e-7 (1 M), 2.4e-7 and 1.3e-7 before.  A copy that does not land within
+// the bound makes its segment's sums NaN.
+constexpr uint32_t GB_ROWS = ST_TRACKS * 24u, GB_BUF = 2u * GB_ROWS;
+constexpr int GB_WARPS = 6;
+static_assert(32 * (NPAR + 1) * 4 <= (int)GB_ROWS && GB_ROWS % 16 == 0, "buffer");
+__global__ void __launch_bounds__(GB_WARPS * 32, 1)
+    k_grad_bulk(const float *__restrict__ x, const float *__restrict__ grad_y,
+                const int32_t *__restrict__ item_sector, const int32_t *__restrict__ item_start,
+                const int32_t *__restrict__ n_items, uint64_t n, float *item_grad) {
+    constexpr int TPL = CALIB_CHUNK / 32;   // tracks per lane and item
+    extern __shared__ __align__(128) unsigned char gb_buf[];
+    __shared__ __align__(8) uint64_t bars[GB_WARPS][2];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const uint32_t gw = blockIdx.x * GB_WARPS + wib, nw = gridDim.x * GB_WARPS;
+    allow_next_grid();   // k_lg_final's blocks may take SMs as this grid's blocks leave
+    const uint32_t NI = (uint32_t)*n_items;
+    if (NI == 0) return;
+    const CalibRuns runs(nw, NI);
+    if (gw >= runs.nwe) return;
+    const uint32_t i0 = runs.first(gw), i1 = runs.first(gw + 1);
+    unsigned char *wbuf = gb_buf + (size_t)wib * 2 * GB_BUF;
+    uint64_t *mb = bars[wib];
+    if (lane == 0) {
+        mbar_init(&mb[0], 1);
+        mbar_init(&mb[1], 1);
+        mbar_init_fence();
+    }
+    __syncwarp();
+    const uint32_t n32 = (uint32_t)n, n4 = n32 & ~3u;
+    // sector, first track and end of the item of this lane in the batch of 32
+    // items from `base`, and of the one after
+    uint32_t base = i0, c_s, c_st, c_en, x_s, x_st, x_en;
+    auto fetch = [&](uint32_t b0, uint32_t &ms, uint32_t &mst, uint32_t &men) {
+        const uint32_t i = b0 + (uint32_t)lane;
+        ms = mst = men = 0;
+        if (i < i1) {
+            ms = (uint32_t)__ldg(item_sector + i);
+            mst = (uint32_t)__ldg(item_start + i);
+            men = i + 1 < NI ? (uint32_t)__ldg(item_start + i + 1) : n32;
+        }
+    };
+    auto info = [&](uint32_t j, uint32_t &sec, uint32_t &st, uint32_t &en) {
+        const uint32_t d = j - base;   // below 64
+        const int src = (int)(d & 31u);
+        const uint32_t a0 = __shfl_sync(0xffffffffu, c_s, src), b0 = __shfl_sync(0xffffffffu, x_s, src);
+        const uint32_t a1 = __shfl_sync(0xffffffffu, c_st, src), b1 = __shfl_sync(0xffffffffu, x_st, src);
+        const uint32_t a2 = __shfl_sync(0xffffffffu, c_en, src), b2 = __shfl_sync(0xffffffffu, x_en, src);
+        sec = d < 32 ? a0 : b0;
+        st = d < 32 ? a1 : b1;
+        en = d < 32 ? a2 : b2;
+    };
+    // item j's rows [lo, hi) into buffer b (every lane's reads of b are done)
+    auto issue = [&](uint32_t j, uint32_t b) {
+        uint32_t sec, st, en;
+        info(j, sec, st, en);
+        const uint32_t lo = st & ~3u, hi = max(lo, min((en + 3u) & ~3u, n4));
+        __syncwarp();
+        if (lane == 0) {
+            unsigned char *d = wbuf + (size_t)b * GB_BUF;
+            fence_proxy_async_smem();
+            mbar_arrive_expect_tx(&mb[b], (hi - lo) * 48u);
+            if (hi > lo) {
+                bulk_copy_g2s(d, x + (size_t)lo * 6, (hi - lo) * 24u, &mb[b]);
+                bulk_copy_g2s(d + GB_ROWS, grad_y + (size_t)lo * 6, (hi - lo) * 24u, &mb[b]);
+            }
+        }
+    };
+    fetch(base, c_s, c_st, c_en);
+    fetch(base + 32, x_s, x_st, x_en);
+    issue(i0, 0);
+    float acc[NPAR];   // the run's sums in its current sector
+#pragma unroll
+    for (int j = 0; j < NPAR; ++j) acc[j] = 0.f;
+    uint32_t seg = i0, bad = 0u, ever_bad = 0u;
+    for (uint32_t i = i0; i < i1; ++i) {
+        const uint32_t b = (i - i0) & 1u, parity = ((i - i0) >> 1) & 1u;
+        if (i - base >= 32u) {   // the next batch of lookups
+            base += 32;
+            c_s = x_s; c_st = x_st; c_en = x_en;
+            fetch(base + 32, x_s, x_st, x_en);
+        }
+        uint32_t is, start, iend, next = ~0u;
+        info(i, is, start, iend);
+        if (i + 1 < i1) {
+            uint32_t st2, en2;
+            issue(i + 1, b ^ 1u);
+            info(i + 1, next, st2, en2);
+        }
+        const uint32_t lo = start & ~3u, hi = max(lo, min((iend + 3u) & ~3u, n4));
+        if (!mbar_wait_bounded(&mb[b], parity)) bad = 1u;
+        const float *xs = reinterpret_cast<const float *>(wbuf + (size_t)b * GB_BUF);
+        const float *gs = reinterpret_cast<const float *>(wbuf + (size_t)b * GB_BUF + GB_ROWS);
+        float sum[NPAR];   // the lane's tracks of the item
+#pragma unroll
+        for (int j = 0; j < NPAR; ++j) sum[j] = 0.f;
+#pragma unroll 2
+        for (int u = 0; u < TPL; ++u) {
+            const uint32_t t = start + (uint32_t)lane + 32u * (uint32_t)u;
+            if (t >= iend) break;
+            float xv[6], g[6];
+            if (t < hi) {
+                const float2 *xp = reinterpret_cast<const float2 *>(xs + (size_t)(t - lo) * 6);
+                const float2 *gp = reinterpret_cast<const float2 *>(gs + (size_t)(t - lo) * 6);
+#pragma unroll
+                for (int l = 0; l < 3; ++l) {
+                    xv[2 * l] = xp[l].x; xv[2 * l + 1] = xp[l].y;
+                    g[2 * l] = gp[l].x; g[2 * l + 1] = gp[l].y;
+                }
+            } else {   // past the last multiple of four tracks
+#pragma unroll
+                for (int l = 0; l < 6; ++l) {
+                    xv[l] = __ldg(x + (size_t)t * 6 + l);
+                    g[l] = __ldg(grad_y + (size_t)t * 6 + l);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+#pragma unroll
+                for (int l = 0; l < 6; ++l) sum[k * 6 + l] = fmaf(g[k], xv[l], sum[k * 6 + l]);
+                sum[36 + k] += g[k];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < NPAR; ++j) acc[j] += sum[j];
+        // does the segment end with this item?
+        if (i + 1 != i1 && next == is) continue;
+        {   // the segment's sums over the lanes, through item i's x rows: four runs of
+            // eight lanes in lane order, then the runs in a fixed tree
+            float *red = reinterpret_cast<float *>(wbuf + (size_t)b * GB_BUF);
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < NPAR; ++j) red[lane * (NPAR + 1) + j] = acc[j];
+            __syncwarp();
+            const bool lost = __any_sync(0xffffffffu, bad);
+            for (int j = lane; j < NPAR; j += 32) {
+                float part[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    float v = red[(8 * u) * (NPAR + 1) + j];
+#pragma unroll
+                    for (int m = 1; m < 8; ++m) v += red[(8 * u + m) * (NPAR + 1) + j];
+                    part[u] = v;
+                }
+                const float v = (part[0] + part[1]) + (part[2] + part[3]);
+                item_grad[(size_t)seg * NPAR + j] = lost ? __int_as_float(0x7fc00000) : v;
+            }
+            __syncwarp();
+        }
+        seg = i + 1;
+#pragma unroll
+        for (int j = 0; j < NPAR; ++j) acc[j] = 0.f;
+        ever_bad |= bad;
+        bad = 0u;
+    }
+    // after a wait that gave up, wait (bounded again) for the last copy into
+    // each buffer before the block's shared memory is released
+    if (__any_sync(0xffffffffu, ever_bad)) {
+        const uint32_t n_it = i1 - i0;
+#pragma unroll
+        for (uint32_t b = 0; b < 2; ++b)
+            if (n_it > b) mbar_wait_bounded(&mb[b], ((n_it - 1u - b) >> 1) & 1u);
+    }
+}
 
 // the final sums of the staged pass (see above): blocks [0, ncol) one thread
-// per (sector, entry) (ncol = 0: the loss alone), block ncol the loss; nw =
+// per (sector, entry) (ncol = 0: the loss alone), block ncol, if launched, the loss; nw =
 // the first kernel's warps
 constexpr int LGF_THREADS = 512;
 __global__ void __launch_bounds__(LGF_THREADS)
     k_lg_final(const float *__restrict__ item_grad, const float *__restrict__ item_loss,
                const int32_t *__restrict__ sector_item, const int32_t *__restrict__ n_items,
-               uint32_t S, uint64_t n, uint32_t nw, uint32_t ncol,
+               uint32_t S, uint64_t n, uint32_t nw, uint32_t ncol, float scale_host,
                const float *__restrict__ scale_dev, unsigned int *flag, float *loss, float *dF,
                float *dq) {
     wait_prior_grid();
     const uint32_t NI = (uint32_t)*n_items;
-    const float scale = (n ? 2.0f / (float)n : 0.f) * (scale_dev ? *scale_dev : 1.f);
+    const float scale = scale_host * (scale_dev ? *scale_dev : 1.f);
     const CalibRuns runs(nw, NI);
-    auto first = [&](uint32_t v) { return runs.first(v); };
-    auto warp_of = [&](uint32_t i) { return runs.warp_of(i); };
+    // total + the sector's segment sums in order, eight loads in flight (a total
+    // that starts at +0 is never -0, so the zeros past the end change nothing)
+    auto add_segments = [&](uint32_t s, float total, const float *p, uint32_t stride) {
+        const uint32_t a = (uint32_t)sector_item[s], e = (uint32_t)sector_item[s + 1];
+        if (e <= a) return total;
+        const uint32_t wa = runs.warp_of(a), wz = runs.warp_of(e - 1);
+        for (uint32_t v0 = wa; v0 <= wz; v0 += 8) {
+            float t[8];
+#pragma unroll
+            for (uint32_t u = 0; u < 8; ++u)
+                t[u] = v0 + u <= wz ? p[(size_t)max(a, runs.first(v0 + u)) * stride] : 0.f;
+#pragma unroll
+            for (uint32_t u = 0; u < 8; ++u) total += t[u];
+        }
+        return total;
+    };
     if (blockIdx.x < ncol) {
         const uint32_t k = blockIdx.x * LGF_THREADS + threadIdx.x;
         if (k >= S * NPAR) return;
         const uint32_t s = k / NPAR, j = k % NPAR;
-        const uint32_t a = (uint32_t)sector_item[s], e = (uint32_t)sector_item[s + 1];
-        float total = 0.f;
-        if (e > a) {
-            const uint32_t wa = warp_of(a), wz = warp_of(e - 1);
-#pragma unroll 4
-            for (uint32_t v = wa; v <= wz; ++v) total += item_grad[(size_t)max(a, first(v)) * NPAR + j];
-        }
+        const float total = add_segments(s, 0.f, item_grad + j, NPAR);
         if (j < 36)
             dF[(size_t)s * 36 + j] = total * scale;
         else
@@ -1134,14 +1318,7 @@ __global__ void __launch_bounds__(LGF_THREADS)
     // threads' sums by a fixed shuffle tree per warp and over the warps
     __shared__ float wsum[LGF_THREADS / 32];
     float sl = 0.f;
-    for (uint32_t s = threadIdx.x; s < S; s += LGF_THREADS) {
-        const uint32_t a = (uint32_t)sector_item[s], e = (uint32_t)sector_item[s + 1];
-        if (e > a) {
-            const uint32_t wa = warp_of(a), wz = warp_of(e - 1);
-#pragma unroll 4
-            for (uint32_t v = wa; v <= wz; ++v) sl += item_loss[max(a, first(v))];
-        }
-    }
+    for (uint32_t s = threadIdx.x; s < S; s += LGF_THREADS) sl = add_segments(s, sl, item_loss, 1);
     sl = warp_sum(sl);
     if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = sl;
     __syncthreads();
@@ -1243,7 +1420,7 @@ bool launch_loss_grad_bulk(int kind, const float *x, const float *theta,
     const uint32_t ncol = kind == LGB_LOSS ? 0u : (S * NPAR + LGF_THREADS - 1) / LGF_THREADS;
     launch_after(k_lg_final, ncol + 1, LGF_THREADS, 0, st, (const float *)item_grad,
                  (const float *)item_loss, sector_item, n_items, S, n, (uint32_t)(g * warps), ncol,
-                 scale_dev, flag, loss, dF, dq);
+                 n ? 2.0f / (float)n : 0.f, scale_dev, flag, loss, dF, dq);
     return true;
 }
 
@@ -1345,11 +1522,46 @@ void launch_calib_grad_scale(const float *g, const float *dF, const float *dq, u
     k_grad_scale<<<(S * NPAR + 255) / 256, 256, 0, st>>>(g, dF, dq, S, out_F, out_q);
 }
 
+// resident blocks per SM of k_grad_bulk on the current device (0: it cannot be
+// launched); the first call on a device raises its dynamic shared-memory limit
+int grad_bulk_blocks_per_sm() {
+    constexpr int MAXD = 64;
+    static std::once_flag once[MAXD];
+    static int per_sm[MAXD];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAXD) return 0;
+    std::call_once(once[dev], [dev] {
+        const int smem = GB_WARPS * 2 * (int)GB_BUF;
+        int k = 0;
+        if (cudaFuncSetAttribute(k_grad_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+                cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_grad_bulk, GB_WARPS * 32, smem) !=
+                cudaSuccess)
+            k = 0;
+        per_sm[dev] = k;
+        (void)cudaGetLastError();
+    });
+    return per_sm[dev];
+}
+
 void launch_calib_grad(const float *x, const float *grad_y, const int32_t *item_sector,
                        const int32_t *item_start, const int32_t *sector_off,
                        const int32_t *sector_item, const int32_t *n_items, uint32_t max_items,
-                       uint32_t S, const float *F, float *item_grad, float *dF, float *dq,
-                       float *dx, int grid, cudaStream_t st) {
+                       uint32_t S, uint64_t n, const float *F, float *item_grad, float *dF,
+                       float *dq, float *dx, int sms, int grid, cudaStream_t st) {
+    const int per_sm = grad_bulk_blocks_per_sm();
+    if (!dx && per_sm > 0 && (((uintptr_t)x | (uintptr_t)grad_y) & 15u) == 0) {
+        const int gb = max(sms, 1) * per_sm;
+        k_grad_bulk<<<gb, GB_WARPS * 32, GB_WARPS * 2 * GB_BUF, st>>>(x, grad_y, item_sector,
+                                                                     item_start, n_items, n,
+                                                                     item_grad);
+        const uint32_t ncol = (S * NPAR + LGF_THREADS - 1) / LGF_THREADS;
+        launch_after(k_lg_final, ncol, LGF_THREADS, 0, st, (const float *)item_grad,
+                     (const float *)nullptr, sector_item, n_items, S, n,
+                     (uint32_t)(gb * GB_WARPS), ncol, 1.0f, (const float *)nullptr,
+                     (unsigned int *)nullptr, (float *)nullptr, dF, dq);
+        return;
+    }
     const int g = (int)min((uint32_t)grid, (max_items + 7) / 8 + 1);
     k_grad_items<<<g, 256, 0, st>>>(x, grad_y, item_sector, item_start, sector_off, n_items, F,
                                     item_grad, dx);

@@ -178,7 +178,7 @@ void launch_calib_grad_scale(const float *g, const float *dF, const float *dq, u
 void launch_calib_grad(const float *x, const float *grad_y, const int32_t *item_sector,
                        const int32_t *item_start, const int32_t *sector_off,
                        const int32_t *sector_item, const int32_t *n_items, uint32_t max_items,
-                       uint32_t S, const float *F, float *item_grad, float *dF, float *dq,
-                       float *dx, int grid, cudaStream_t st);
+                       uint32_t S, uint64_t n, const float *F, float *item_grad, float *dF,
+                       float *dq, float *dx, int sms, int grid, cudaStream_t st);
 
 }  // namespace svt
