@@ -157,6 +157,8 @@ _lock = threading.Lock()
 def load():
     """Load libsvt.so (building it first when nvcc is available)."""
     global _lib
+    if _lib is not None:   # once it is there, no call takes the lock
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

@@ -10,8 +10,6 @@ The integer path is untouched by all of this.
 """
 from __future__ import annotations
 
-import ctypes
-
 import numpy as np
 import torch
 
@@ -20,7 +18,13 @@ from .api import _p, _stream
 
 
 def _f32(t):
-    return t.detach().to(torch.float32).contiguous()
+    t = t.detach()
+    return t if t.dtype is torch.float32 and t.is_contiguous() else t.to(torch.float32).contiguous()
+
+
+def _upstream(g):
+    """The gradient of a scalar result as one float32 on the device."""
+    return g if g.dtype is torch.float32 else g.to(torch.float32)
 
 
 class CalibData:
@@ -63,14 +67,15 @@ class FitFP32(torch.autograd.Function):
                                     _p(q32), _p(y), _stream(None)), "svt_calib_forward")
         ctx.data = data
         ctx.save_for_backward(F32)
-        return y[: data.n]
+        return y if data.n else y[:0]
 
     @staticmethod
     def backward(ctx, gy):
         L = N.load()
         data = ctx.data
         (F32,) = ctx.saved_tensors
-        gy = gy.to(torch.float32).contiguous()
+        if gy.dtype is not torch.float32 or not gy.is_contiguous():
+            gy = gy.to(torch.float32).contiguous()
         dF = torch.empty_like(F32)
         dq = torch.empty((data.n_sectors, 6), dtype=torch.float32, device=F32.device)
         N.check(L.svt_calib_backward(_p(data.x), _p(gy), data.n, data.n_sectors, _p(data.index),
@@ -91,7 +96,7 @@ class CalibLoss(torch.autograd.Function):
     def forward(ctx, F, q, data: CalibData):
         L = N.load()
         F32, q32 = _f32(F), _f32(q)
-        loss = torch.empty(1, dtype=torch.float32, device=F.device)
+        loss = torch.empty((), dtype=torch.float32, device=F.device)
         ctx.data = data
         if ctx.needs_input_grad[0] or ctx.needs_input_grad[1]:
             dF = torch.empty_like(F32)
@@ -107,13 +112,13 @@ class CalibLoss(torch.autograd.Function):
                                      data.n_sectors, _p(data.index), _p(F32), _p(q32), _p(loss),
                                      _p(data.workspace), data.workspace.numel(), _stream(None)),
                     "svt_calib_loss")
-        return loss[0]
+        return loss
 
     @staticmethod
     def backward(ctx, gL):
         L = N.load()
         dF, dq = ctx.saved_tensors
-        g = gL.to(torch.float32).contiguous().reshape(1)
+        g = _upstream(gL)
         out_F = torch.empty_like(dF)
         out_q = torch.empty_like(dq)
         N.check(L.svt_calib_grad_scale(_p(g), _p(dF), _p(dq), ctx.data.n_sectors, _p(out_F),
@@ -131,20 +136,20 @@ class CalibLossUnfused(torch.autograd.Function):
     def forward(ctx, F, q, data: CalibData):
         L = N.load()
         F32, q32 = _f32(F), _f32(q)
-        loss = torch.empty(1, dtype=torch.float32, device=F.device)
+        loss = torch.empty((), dtype=torch.float32, device=F.device)
         N.check(L.svt_calib_loss(_p(data.x), _p(data.theta), _p(data.w), data.n, data.n_sectors,
                                  _p(data.index), _p(F32), _p(q32), _p(loss), _p(data.workspace),
                                  data.workspace.numel(), _stream(None)), "svt_calib_loss")
         ctx.data = data
         ctx.save_for_backward(F32, q32)
-        return loss[0]
+        return loss
 
     @staticmethod
     def backward(ctx, gL):
         L = N.load()
         data = ctx.data
         F32, q32 = ctx.saved_tensors
-        g = gL.to(torch.float32).contiguous().reshape(1)
+        g = _upstream(gL)
         dF = torch.empty_like(F32)
         dq = torch.empty_like(q32)
         N.check(L.svt_calib_loss_backward(_p(data.x), _p(data.theta), _p(data.w), data.n,
@@ -165,7 +170,7 @@ class CalibLossFit(torch.autograd.Function):
     def forward(ctx, F, q, data: CalibData):
         L = N.load()
         F32, q32 = _f32(F), _f32(q)
-        loss = torch.empty(1, dtype=torch.float32, device=F.device)
+        loss = torch.empty((), dtype=torch.float32, device=F.device)
         y = torch.empty((max(data.n, 1), 6), dtype=torch.float32, device=F.device)
         dF = torch.empty_like(F32)
         dq = torch.empty_like(q32)
@@ -176,9 +181,9 @@ class CalibLossFit(torch.autograd.Function):
                 "svt_calib_loss_grad")
         ctx.data = data
         ctx.save_for_backward(dF, dq)
-        y = y[: data.n]
+        y = y if data.n else y[:0]
         ctx.mark_non_differentiable(y)
-        return loss[0], y
+        return loss, y
 
     @staticmethod
     def backward(ctx, gL, gy):

@@ -50,12 +50,14 @@ class Server:
     def submit(self, h_words: torch.Tensor, tag: int, h_records: np.ndarray | None = None) -> int:
         """Queue one event whose words are a pinned host tensor (kept alive
         until its result arrives).  Returns the C status code."""
-        rec = None if h_records is None else h_records.ctypes.data_as(ctypes.c_void_p)
-        return N.load().svt_server_submit(self.handle, ctypes.c_void_p(h_words.data_ptr()),
-                                          h_words.numel(), tag, rec)
+        rec = None if h_records is None else h_records.ctypes.data
+        return N.load().svt_server_submit(self.handle, h_words.data_ptr(), h_words.numel(), tag, rec)
 
     def poll(self, max_results=4096, wait_us=1000):
-        buf = (N.SvtEventResult * max_results)()
+        # memory that is not cleared first (196 KB at the default, which cost
+        # more than the rest of the call); the results returned keep it alive
+        buf = (N.SvtEventResult * max_results).from_buffer(
+            np.empty(max_results * ctypes.sizeof(N.SvtEventResult), np.uint8))
         n = ctypes.c_uint32()
         N.check(N.load().svt_server_poll(self.handle, buf, max_results, ctypes.byref(n), wait_us),
                 "svt_server_poll")
