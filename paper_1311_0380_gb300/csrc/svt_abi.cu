@@ -239,7 +239,7 @@ int svt_unpack(const uint32_t *d_words, uint64_t n_words, const uint64_t *d_even
     const FusedRoads none{nullptr, nullptr, BigList{}, 1, 0};
     launch_unpack_roads(d_words, d_event_off, w.dims, w.first_ev, n_words, w.tile_state,
                         w.tile_ticket, d_n_roads, road_cap, d_road_word, d_road_nhit, d_event_road,
-                        cfg, none, nullptr, status, grid, st);
+                        cfg, none, nullptr, status, grid, false, st);
     launch_unpack_events(d_words, d_event_off, w.dims, n_events, d_event_road, status, grid, st);
     return launch_status();
 }
@@ -369,7 +369,7 @@ int run_impl(const uint32_t *d_words, uint64_t n_words, const uint64_t *d_event_
                         w.work, 2, w.tile_state, w.tile_ticket, grid, st);
         launch_unpack_roads(d_words, d_event_off, w.dims, w.first_ev, n_words, w.tile_state,
                             w.tile_ticket, counts + 0, road_cap, nullptr, nullptr, event_road,
-                            *cfg, fr, counts, status, grid, st);
+                            *cfg, fr, counts, status, grid, fit_group(sc.pair_small) == 32, st);
     }
     const NvtxRange fit_range("svt_run: combine, fit, cut, select, format");
     if (timer && cudaEventRecord(timer->start, st) != cudaSuccess) return SVT_ERR_CUDA;

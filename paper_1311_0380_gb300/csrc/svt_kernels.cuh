@@ -32,20 +32,29 @@ __device__ __forceinline__ void allow_next_grid() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// max_shared: the SMs' on-chip memory is split for as much shared memory as
+// there is, not just what this kernel needs.
 template <typename... KArgs, typename... Args>
-inline void launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                         cudaStream_t st, Args... args) {
-    cudaLaunchAttribute attr[1];
+inline void launch_chained(bool max_shared, void (*kernel)(KArgs...), dim3 grid, dim3 block,
+                           size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
     cudaLaunchConfig_t c = {};
     c.gridDim = grid;
     c.blockDim = block;
     c.dynamicSmemBytes = smem;
     c.stream = st;
     c.attrs = attr;
-    c.numAttrs = 1;
+    c.numAttrs = max_shared ? 2 : 1;
     cudaLaunchKernelEx(&c, kernel, args...);   // errors surface through cudaGetLastError
+}
+template <typename... KArgs, typename... Args>
+inline void launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                         cudaStream_t st, Args... args) {
+    launch_chained(false, kernel, grid, block, smem, st, args...);
 }
 
 // ---- unpack (svt_unpack.cu) --------------------------------------------------
@@ -71,7 +80,8 @@ void launch_unpack_roads(const uint32_t *words, const uint64_t *event_off, const
                          unsigned long long *tile_state, uint32_t *tile_ticket, uint64_t *total64,
                          uint64_t road_cap, uint32_t *road_word, uint32_t *road_nhit,
                          uint32_t *event_road, const svt_config cfg, const FusedRoads fr,
-                         uint64_t *counts, unsigned long long *status, int grid, cudaStream_t st);
+                         uint64_t *counts, unsigned long long *status, int grid, bool max_shared,
+                         cudaStream_t st);
 // Per-event rules of the plain path: offsets and V10.
 void launch_unpack_events(const uint32_t *words, const uint64_t *event_off, const Dims *dims,
                           uint64_t max_events, const uint32_t *event_road,
