@@ -132,7 +132,8 @@ typedef struct {
  *                    work item of a split road (1..1024, default 16; each
  *                    item repeats its road's set-up, so longer items cost
  *                    less set-up and balance the work less finely)
- *   roads_per_chunk  consecutive roads a warp takes at once (1..32, default 4)
+ *   roads_per_chunk  consecutive roads a warp takes at once (1..32, default 4; with
+ *                    pair_small 0 the last two roads per warp come one by one)
  *   small_max        roads with more evaluated combinations than this are
  *                    split into work items; the others are fitted whole by
  *                    one warp (default 4096)

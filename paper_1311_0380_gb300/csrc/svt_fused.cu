@@ -1407,6 +1407,26 @@ __device__ __forceinline__ uint32_t flush_records(const uint32_t *__restrict__ w
     return n_pass;
 }
 
+// Chunks of consecutive roads that the warps claim (GROUP 1): roads_per_chunk
+// roads each, but single roads for the last GUIDED_TAIL roads per warp, so that
+// the warps finish together and a batch of few roads spreads over all of them,
+// while a large batch does not queue on the counter (0.7 ns a claim).  Whole
+// passes with chunks of 4 throughout and like this: scaled shape, 100 events
+// 37.2 and 30.9 us, 3000 events 205.2 and 204.6; 1000 paired events 75.6 and
+// 74.0; with single roads throughout 29.9, 211.8 and 80.7.  A tail of 1 road per
+// warp leaves 100 events at 34.8, one of 4 costs 3 % for 32,000 short roads.
+// (First claims handed out without the counter, or one counter for items and
+// chunks, are 2 us faster for 100 events and 1-15 % slower for large batches.)
+constexpr uint32_t GUIDED_TAIL = 2;
+__device__ __forceinline__ uint32_t full_chunks(uint32_t R, uint32_t per, uint32_t warps) {
+    return (R - min(R, GUIDED_TAIL * warps)) / per;
+}
+// the first road of chunk k (R or more: there is no such chunk)
+__device__ __forceinline__ uint32_t chunk_first(uint32_t k, uint32_t n_full, uint32_t per,
+                                                uint32_t R) {
+    return k < n_full ? k * per : n_full * per + min(k - n_full, R);
+}
+
 // The fit of a whole batch by screening: items of split roads, then chunks of
 // consecutive roads, each road by one warp.  Returns the passing roads whose
 // records this lane wrote.
@@ -1424,7 +1444,7 @@ __device__ __forceinline__ uint32_t screen_path(
         n_pass += flush_records(words, desc, F, q, cfg, out, rl, slot.flush, n_rec);
         n_rec = 0;
     };
-    for (;;) {
+    while (n_items) {   // (no items: no claim, 3.5 us of queueing for a grid's warps)
         uint32_t it = 0;
         if (lane == 0) it = atomicAdd(bl.counters + 0, 1u);
         it = __shfl_sync(0xffffffffu, it, 0);
@@ -1462,13 +1482,14 @@ __device__ __forceinline__ uint32_t screen_path(
         }
         __syncwarp();
     }
+    const uint32_t n_full = full_chunks(R, roads_per_chunk, gridDim.x * (blockDim.x >> 5));
     for (;;) {
         uint32_t k = 0;
         if (lane == 0) k = atomicAdd(bl.counters + 1, 1u);
         k = __shfl_sync(0xffffffffu, k, 0);
-        if ((uint64_t)k * roads_per_chunk >= R) break;
-        const uint32_t c0 = k * roads_per_chunk;
-        const uint32_t n = min(roads_per_chunk, R - c0);
+        const uint32_t c0 = chunk_first(k, n_full, roads_per_chunk, R);
+        if (c0 >= R) break;
+        const uint32_t n = k < n_full ? roads_per_chunk : 1u;
         uint4 da = make_uint4(0, 0, 0, 0), db = make_uint4(0, 0, 0, 0);
         if ((uint32_t)lane < n) {
             da = __ldg(&desc[c0 + lane].a);
@@ -1600,7 +1621,8 @@ __global__ void __launch_bounds__(GROUP == 32 ? 384 : 512, 2)
     const bool static_first = (GROUP == 4 || GROUP == 32) && n_items == 0;
 
     // phase 1: items of split roads
-    while (!static_first) {
+    // (GROUP 1: none, no claim: a grid's warps queue 3.5 us on one counter)
+    while (GROUP == 1 ? n_items != 0 : !static_first) {
         uint32_t it = 0;
         if (lane == 0) it = atomicAdd(bl.counters + 0, 1u);
         it = __shfl_sync(0xffffffffu, it, 0);
@@ -1638,14 +1660,25 @@ __global__ void __launch_bounds__(GROUP == 32 ? 384 : 512, 2)
     // phase 2: chunks of consecutive roads, each fitted whole by this warp,
     // or two SMALL roads side by side by its two halves
     for (bool first = true;; first = false) {
-        uint32_t k = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;   // chunk index
-        if (!(first && static_first)) {
-            if (lane == 0) k = atomicAdd(bl.counters + 1, 1u) + (static_first ? nw : 0u);
+        uint32_t c0, n;
+        if constexpr (GROUP == 1) {
+            uint32_t k = 0;
+            if (lane == 0) k = atomicAdd(bl.counters + 1, 1u);
             k = __shfl_sync(0xffffffffu, k, 0);
+            const uint32_t full = full_chunks(R, roads_per_chunk, nw);
+            c0 = chunk_first(k, full, roads_per_chunk, R);
+            if (c0 >= R) break;
+            n = k < full ? roads_per_chunk : 1u;
+        } else {
+            uint32_t k = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;   // chunk index
+            if (!(first && static_first)) {
+                if (lane == 0) k = atomicAdd(bl.counters + 1, 1u) + (static_first ? nw : 0u);
+                k = __shfl_sync(0xffffffffu, k, 0);
+            }
+            if ((uint64_t)k * roads_per_chunk >= R) break;
+            c0 = k * roads_per_chunk;
+            n = min(roads_per_chunk, R - c0);
         }
-        if ((uint64_t)k * roads_per_chunk >= R) break;
-        const uint32_t c0 = k * roads_per_chunk;
-        const uint32_t n = min(roads_per_chunk, R - c0);
         // this lane's road of the chunk (GROUP 32: L lanes to a road)
         const uint32_t jr = (uint32_t)lane / L;
         uint4 da = make_uint4(0, 0, 0, 0), db = make_uint4(0, 0, 0, 0);
