@@ -279,23 +279,52 @@ __global__ void __launch_bounds__(WRITE_THREADS)
     }
 }
 
-// acc_k = q_k 2^qshift + sum_l F_kl x_l exactly, with 32-bit products:
-// |F_kl x_l| <= 32768 * 32767 < 2^30, so every sum of two products is exact
-// in int32; the three pair sums and q_k 2^qshift (|.| < 2^39) are added in
-// int64.  With oshift >= 9, |y_k| < 2^31 and y_k = floor(acc_k / 2^oshift) is
-// exact in int32.  Results: chi2 over the three clamped chi rows, p_0..p_2.
-__device__ __forceinline__ uint32_t fit_rows(const int32_t (&Fk)[36], const long long (&qk)[6],
-                                             const int32_t (&x)[N_LAYERS], uint32_t oshift,
-                                             int32_t (&p)[3]) {
+// A constant row as the fit takes it: F in pairs of 16 bits (F_k,2m low), and
+// Q_k = q_k 2^qshift as its low nine bits and the rest (|Q_k| < 2^39).
+struct PackedRow {
+    int32_t F[18];
+    int32_t q_lo[6], q_hi[6];
+};
+__device__ __forceinline__ int32_t pack_pair(int16_t lo, int16_t hi) {
+    return (int32_t)((uint32_t)(uint16_t)lo | ((uint32_t)(uint16_t)hi << 16));
+}
+__device__ __forceinline__ long long shifted_q(int16_t q, uint32_t qshift) {
+    return (long long)((unsigned long long)(long long)q << qshift);
+}
+// c + a.lo b.byte0 + a.hi b.byte1, and the same with bytes 2 and 3
+__device__ __forceinline__ int32_t dot_lo(int32_t a, uint32_t b, int32_t c) {
+    int32_t d;
+    asm("dp2a.lo.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+__device__ __forceinline__ int32_t dot_hi(int32_t a, uint32_t b, int32_t c) {
+    int32_t d;
+    asm("dp2a.hi.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
+// y_k = floor((Q_k + sum_l F_kl x_l) / 2^oshift) exactly, in 32 bits: with
+// x_l = 256 h_l + b_l (x_l < 2^15) the sum is A + 256 B, A and B dot products of
+// 16-bit constants and bytes (|A|, |B| < 2^26, two terms an instruction), and
+// with Q_k = 512 q_hi + q_lo and oshift >= 9
+//   y_k = floor((q_hi + floor((floor((A + q_lo) / 256) + B) / 2)) / 2^(oshift - 9)).
+// (Sums of 32-bit products in int64, with rows of half as many constants a word,
+// kept the integer pipe 70 % busy: 208 instructions a combination.  7.4 M
+// combinations: 56.2 us then, 48.9 now, 26 for the bytes.)  Results: chi2 over
+// the three clamped chi rows, p_0..p_2.
+__device__ __forceinline__ uint32_t fit_rows(const PackedRow &row, const uint32_t (&x)[N_LAYERS],
+                                             uint32_t oshift, int32_t (&p)[3]) {
+    const uint32_t x01 = __byte_perm(x[0], x[1], 0x5410), x23 = __byte_perm(x[2], x[3], 0x5410);
+    const uint32_t b03 = __byte_perm(x01, x23, 0x6420), h03 = __byte_perm(x01, x23, 0x7531);
+    // b_4, b_5, h_4, h_5
+    const uint32_t x45 = __byte_perm(x[4], x[5], 0x5140);
     int32_t y[N_LAYERS];
 #pragma unroll
     for (int k = 0; k < N_LAYERS; ++k) {
-        int32_t s2[3];
-#pragma unroll
-        for (int m = 0; m < 3; ++m)
-            s2[m] = Fk[k * 6 + 2 * m] * x[2 * m] + Fk[k * 6 + 2 * m + 1] * x[2 * m + 1];
-        const long long acc = qk[k] + (long long)s2[0] + (long long)s2[1] + (long long)s2[2];
-        y[k] = (int32_t)(acc >> oshift);   // arithmetic shift: floor
+        const int32_t *Fk = row.F + 3 * k;
+        int32_t v = dot_lo(Fk[2], x45, dot_hi(Fk[1], b03, dot_lo(Fk[0], b03, row.q_lo[k])));
+        v = dot_hi(Fk[2], x45, dot_hi(Fk[1], h03, dot_lo(Fk[0], h03, v >> 8)));
+        y[k] = (row.q_hi[k] + (v >> 1)) >> (oshift - 9u);
     }
     uint32_t chi2 = 0;
 #pragma unroll
@@ -321,77 +350,75 @@ __device__ __forceinline__ uint32_t fit_direct(const uint32_t *__restrict__ word
     const uint32_t packed = __ldg(road_nhit + r);
     const uint32_t hw = __ldg(words + rw);
     uint32_t mask = 0, hoff = rw + 1;
-    int32_t x[N_LAYERS];
+    uint32_t x[N_LAYERS];
 #pragma unroll
     for (int l = 0; l < N_LAYERS; ++l) {
         const uint32_t nl = nhit_of(packed, l);
-        x[l] = nl ? (int32_t)hit_coord(__ldg(words + hoff + ((hits >> (4 * l)) & 15u))) : 0;
+        x[l] = nl ? hit_coord(__ldg(words + hoff + ((hits >> (4 * l)) & 15u))) : 0u;
         mask |= nl ? (1u << l) : 0u;
         hoff += nl;
     }
     const size_t cs = (size_t)rd_sector(hw) * 64 + mask;
-    int32_t Fk[36];
-    long long qk[6];
+    PackedRow row;
 #pragma unroll
-    for (int i = 0; i < 36; ++i) Fk[i] = __ldg(F + cs * 36 + i);
+    for (int i = 0; i < 18; ++i)
+        row.F[i] = pack_pair(__ldg(F + cs * 36 + 2 * i), __ldg(F + cs * 36 + 2 * i + 1));
 #pragma unroll
-    for (int k = 0; k < 6; ++k)
-        qk[k] = (long long)((unsigned long long)(long long)__ldg(q + cs * 6 + k) << cfg.qshift);
-    return fit_rows(Fk, qk, x, cfg.oshift, p);
+    for (int k = 0; k < 6; ++k) {
+        const long long Q = shifted_q(__ldg(q + cs * 6 + k), cfg.qshift);
+        row.q_lo[k] = (int32_t)(Q & 511);
+        row.q_hi[k] = (int32_t)(Q >> 9);
+    }
+    return fit_rows(row, x, cfg.oshift, p);
 }
 
-// A road's row staged in shared memory by the plain fit: its constants as
-// int32, q_k 2^qshift as int64 and, per layer, the index of its first hit in
-// the road's coordinate list (0xFF for a layer without hits); the road's hit
-// coordinates sit beside it (at most 96: 6 layers x 16).
+// A road's row staged in shared memory by the plain fit: its constants and, per
+// layer, the index of its first hit in the road's coordinate list (0xFF for a
+// layer without hits); the road's hit coordinates sit beside it (at most 96: 6
+// layers x 16).
 constexpr int FIT_THREADS = 256;
 constexpr int FIT_PER_THREAD = 8;
 constexpr int FIT_TILE = FIT_THREADS * FIT_PER_THREAD;   // combinations per block tile
 constexpr int FIT_STAGE_ROADS = 64;   // tiles over more roads read their inputs directly
 struct alignas(16) StagedRow {
-    int32_t F[36];
-    long long q[6];
+    PackedRow row;
     uint8_t first[8];
-    uint32_t pad[2];
 };
+static_assert(sizeof(StagedRow) == 128 && sizeof(PackedRow) == 120, "read as eight 16-byte words");
 
 __device__ __forceinline__ uint32_t fit_staged(const StagedRow &row,
                                                const uint16_t *__restrict__ coord,
                                                uint32_t oshift, uint32_t hits, int32_t (&p)[3]) {
-    const uint2 fw = *reinterpret_cast<const uint2 *>(row.first);
-    int32_t x[N_LAYERS];
+    uint4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4 *>(&row)[i];
+    PackedRow r;
+    const uint32_t *const w = reinterpret_cast<const uint32_t *>(v);
+#pragma unroll
+    for (int i = 0; i < 18; ++i) r.F[i] = (int32_t)w[i];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        r.q_lo[k] = (int32_t)w[18 + k];
+        r.q_hi[k] = (int32_t)w[24 + k];
+    }
+    uint32_t x[N_LAYERS];
 #pragma unroll
     for (int l = 0; l < N_LAYERS; ++l) {
-        const uint32_t f0 = ((l < 4 ? fw.x : fw.y) >> (8 * (l & 3))) & 0xFFu;
-        x[l] = f0 != 0xFFu ? (int32_t)coord[f0 + ((hits >> (4 * l)) & 15u)] : 0;
+        const uint32_t f0 = (w[30 + l / 4] >> (8 * (l & 3))) & 0xFFu;
+        x[l] = f0 != 0xFFu ? coord[f0 + ((hits >> (4 * l)) & 15u)] : 0u;
     }
-    int32_t Fk[36];
-    long long qk[6];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const int4 v = reinterpret_cast<const int4 *>(row.F)[i];
-        Fk[4 * i] = v.x;
-        Fk[4 * i + 1] = v.y;
-        Fk[4 * i + 2] = v.z;
-        Fk[4 * i + 3] = v.w;
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const longlong2 v = reinterpret_cast<const longlong2 *>(row.q)[i];
-        qk[2 * i] = v.x;
-        qk[2 * i + 1] = v.y;
-    }
-    return fit_rows(Fk, qk, x, oshift, p);
+    return fit_rows(r, x, oshift, p);
 }
 
 // One thread per combination, over block tiles of FIT_TILE consecutive
 // combinations (thread t takes combinations t, t + 256, t + 512, ... of the
-// tile and loads their entries first; 48 registers leave five blocks per SM).  Combinations are road-major, so a
+// tile and loads their entries first; six blocks per SM, 48.9 us for 7.4 M
+// combinations, with five 50.1, with three 54.1).  Combinations are road-major, so a
 // tile covers the roads comb_road[first] .. comb_road[last]; when there are
 // at most FIT_STAGE_ROADS of them, their rows and hit coordinates are staged
 // in shared memory once (coalesced loads) and the combinations of the tile
 // need no other global load; otherwise each reads its inputs directly.
-__global__ void __launch_bounds__(FIT_THREADS, 5)
+__global__ void __launch_bounds__(FIT_THREADS, 6)
     k_fit_plain(const uint32_t *__restrict__ words, const uint32_t *__restrict__ road_word,
                 const uint32_t *__restrict__ road_nhit, const uint32_t *__restrict__ comb_road,
                 const uint32_t *__restrict__ comb_hits, const uint64_t *__restrict__ n_combs,
@@ -424,9 +451,9 @@ __global__ void __launch_bounds__(FIT_THREADS, 5)
         const uint32_t r0 = tile_r0, nr = tile_nr;
         const bool staged = nr <= (uint32_t)FIT_STAGE_ROADS;
         if (staged) {
-            // warp w stages roads w, w + 8, ...: lane i of the F row (lanes
-            // 0..3 twice), lanes 4..9 the q row, lanes 10..15 the layers, and
-            // every lane some of the hit coordinates
+            // warp w stages roads w, w + 8, ...: lanes 0..17 the F row, 18..23
+            // the q row, 24..29 the layers, and every lane some of the hit
+            // coordinates
             for (uint32_t rho = warp; rho < nr; rho += FIT_THREADS / 32) {
                 const uint32_t r = r0 + rho;
                 const uint32_t rw = __ldg(road_word + r), packed = __ldg(road_nhit + r);
@@ -439,15 +466,16 @@ __global__ void __launch_bounds__(FIT_THREADS, 5)
                 total = min(total, (uint32_t)(N_LAYERS * MAX_HITS));
                 const size_t cs = (size_t)rd_sector(__ldg(words + rw)) * 64 + mask;
                 StagedRow &row = rows[rho];
-                row.F[lane] = __ldg(F + cs * 36 + lane);
-                if (lane < 4) {
-                    row.F[32 + lane] = __ldg(F + cs * 36 + 32 + lane);
-                } else if (lane < 10) {
-                    const int k = lane - 4;
-                    row.q[k] = (long long)((unsigned long long)(long long)__ldg(q + cs * 6 + k)
-                                           << cfg.qshift);
-                } else if (lane < 16) {
-                    const int l = lane - 10;
+                if (lane < 18) {
+                    row.row.F[lane] = pack_pair(__ldg(F + cs * 36 + 2 * lane),
+                                                __ldg(F + cs * 36 + 2 * lane + 1));
+                } else if (lane < 24) {
+                    const int k = lane - 18;
+                    const long long Q = shifted_q(__ldg(q + cs * 6 + k), cfg.qshift);
+                    row.row.q_lo[k] = (int32_t)(Q & 511);
+                    row.row.q_hi[k] = (int32_t)(Q >> 9);
+                } else if (lane < 24 + N_LAYERS) {
+                    const int l = lane - 24;
                     uint32_t before = 0;   // hits on the layers below l
 #pragma unroll
                     for (int m = 0; m < N_LAYERS - 1; ++m) before += m < l ? nhit_of(packed, m) : 0u;
