@@ -75,6 +75,14 @@ uint32_t fit_group(uint32_t pair_small) {
     return pair_small == 3 ? 32u : pair_small == 2 ? 4u : pair_small == 1 ? 2u : 1u;
 }
 
+// whether p is device memory (not mapped or unregistered host memory)
+bool in_device_memory(const void *p) {
+    cudaPointerAttributes a;
+    if (p && cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type == cudaMemoryTypeDevice;
+    if (p) (void)cudaGetLastError();
+    return false;
+}
+
 int launch_status() {
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? SVT_OK : SVT_ERR_CUDA;
@@ -369,7 +377,8 @@ int run_impl(const uint32_t *d_words, uint64_t n_words, const uint64_t *d_event_
                         w.work, 2, w.tile_state, w.tile_ticket, grid, st);
         launch_unpack_roads(d_words, d_event_off, w.dims, w.first_ev, n_words, w.tile_state,
                             w.tile_ticket, counts + 0, road_cap, nullptr, nullptr, event_road,
-                            *cfg, fr, counts, status, grid, fit_group(sc.pair_small) == 32, st);
+                            *cfg, fr, counts, status, grid,
+                            fit_group(sc.pair_small) == 32 && in_device_memory(d_words), st);
     }
     const NvtxRange fit_range("svt_run: combine, fit, cut, select, format");
     if (timer && cudaEventRecord(timer->start, st) != cudaSuccess) return SVT_ERR_CUDA;

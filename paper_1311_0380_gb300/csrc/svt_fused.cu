@@ -1512,9 +1512,11 @@ __device__ __forceinline__ uint32_t screen_path(
     return n_pass;
 }
 
-constexpr size_t LIST_BYTES =
-    sizeof(RecordList) > sizeof(CandList) ? sizeof(RecordList) : sizeof(CandList);
-static_assert(LIST_BYTES % 16 == 0, "lists keep 16-byte alignment");
+// a warp's list beside its slot (GROUP 1 screens and lists candidates as well)
+template <int GROUP>
+constexpr size_t LIST_BYTES = GROUP == 1 && sizeof(CandList) > sizeof(RecordList)
+                                  ? sizeof(CandList) : sizeof(RecordList);
+static_assert(LIST_BYTES<1> % 16 == 0 && LIST_BYTES<32> % 16 == 0, "lists keep 16-byte alignment");
 // Mean evaluated combinations of a batch's roads from which on the batch is
 // fitted by screening (one road per warp, GROUP 1; one form per launch, so that
 // the warps keep to one path of code).  Its set-up, listing and exact step cost
@@ -1552,7 +1554,7 @@ __global__ void __launch_bounds__(GROUP == 32 ? 384 : 512, 2)
                      uint32_t roads_per_chunk, uint32_t *out, unsigned long long *status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     WarpSmem &sm = *reinterpret_cast<WarpSmem *>(smem_raw + SLOT_BYTES * (threadIdx.x >> 5));
-    unsigned char *list = smem_raw + SLOT_BYTES * (blockDim.x >> 5) + LIST_BYTES * (threadIdx.x >> 5);
+    unsigned char *list = smem_raw + SLOT_BYTES * (blockDim.x >> 5) + LIST_BYTES<GROUP> * (threadIdx.x >> 5);
     RecordList &rl = *reinterpret_cast<RecordList *>(list);
     const int lane = threadIdx.x & 31;
     const Lanes<32> LW = lanes_of<32>(lane);
@@ -1815,8 +1817,8 @@ __global__ void __launch_bounds__(GROUP == 32 ? 384 : 512, 2)
 
 }  // namespace
 
-size_t fit_smem_bytes(int warps_per_block) {
-    return (SLOT_BYTES + LIST_BYTES) * (size_t)warps_per_block;
+size_t fit_smem_bytes(int warps_per_block, uint32_t group) {
+    return (SLOT_BYTES + (group == 1 ? LIST_BYTES<1> : LIST_BYTES<32>)) * (size_t)warps_per_block;
 }
 
 namespace {
@@ -1839,7 +1841,7 @@ Screen make_screen(const svt_config &cfg) {
 
 
 int fit_persistent_blocks_per_sm(int warps_per_block, uint32_t group) {
-    const size_t smem = fit_smem_bytes(warps_per_block);
+    const size_t smem = fit_smem_bytes(warps_per_block, group);
     int occ = 1 << 30;
     auto one = [&](auto kernel) {
         int n = 0;
@@ -1873,7 +1875,7 @@ cudaError_t launch_fit_persistent(const uint32_t *words, const uint64_t *event_o
                                   const FusedRoads fr, uint32_t roads_per_chunk, uint32_t group,
                                   uint32_t *out, unsigned long long *status,
                                   int warps_per_block, int grid, cudaStream_t st) {
-    const size_t smem = fit_smem_bytes(warps_per_block);
+    const size_t smem = fit_smem_bytes(warps_per_block, group);
     const bool guarded = cfg.chi2_cut < SAT;
     const Screen sc = make_screen(cfg);
     auto launch = [&](auto kernel) {

@@ -80,8 +80,8 @@ void launch_unpack_roads(const uint32_t *words, const uint64_t *event_off, const
                          unsigned long long *tile_state, uint32_t *tile_ticket, uint64_t *total64,
                          uint64_t road_cap, uint32_t *road_word, uint32_t *road_nhit,
                          uint32_t *event_road, const svt_config cfg, const FusedRoads fr,
-                         uint64_t *counts, unsigned long long *status, int grid, bool max_shared,
-                         cudaStream_t st);
+                         uint64_t *counts, unsigned long long *status, int grid,
+                         bool max_shared, cudaStream_t st);
 // Per-event rules of the plain path: offsets and V10.
 void launch_unpack_events(const uint32_t *words, const uint64_t *event_off, const Dims *dims,
                           uint64_t max_events, const uint32_t *event_road,
@@ -127,7 +127,7 @@ cudaError_t launch_fit_persistent(const uint32_t *words, const uint64_t *event_o
 // persistent blocks of the fit kernel per SM for a block size and a road
 // grouping (1, 2, 4 or 32; both chi2-cut instances of it)
 int fit_persistent_blocks_per_sm(int warps_per_block, uint32_t group);
-size_t fit_smem_bytes(int warps_per_block);
+size_t fit_smem_bytes(int warps_per_block, uint32_t group);
 
 // ---- plain path (svt_plain.cu) --------------------------------------------------
 // Every plain-path kernel returns at once when *status already holds an error.

@@ -209,7 +209,11 @@ __global__ void __launch_bounds__(TILE_THREADS, 12)
     // hits [31:20].  A field can only overflow in a run of more than 1023 hits,
     // which then also shows more than 96 hits and is not checked.
     __shared__ __align__(16) uint32_t cnt45[PAIR ? TILE_WORDS : 4];
-    __shared__ uint2 hdr[TILE_WORDS];   // each road header: tile position, word
+    // each road header: tile position and word (apart for pairing, whose counts
+    // would otherwise leave twelve tiles no L1)
+    __shared__ uint2 hdr[PAIR ? 1 : TILE_WORDS];
+    __shared__ uint32_t hdr_word[PAIR ? TILE_WORDS : 1];
+    __shared__ uint16_t hdr_pos[PAIR ? TILE_WORDS : 1];
     __shared__ __align__(16) uint32_t hit_bits[ROWS], road_bits[ROWS];
     __shared__ uint32_t event_bits[ROWS];                // (the reserved type as well)
     __shared__ uint32_t same_bits[1 + ROWS];             // [0]: the 32 words before the tile
@@ -376,8 +380,14 @@ __global__ void __launch_bounds__(TILE_THREADS, 12)
                 const uint32_t sm = __ballot_sync(ALL, same);
                 if (lane == 0) same_bits[1 + warp * WARP_ROWS + i] = sm;
                 const int r = r_row + __popc(rm & lt);   // latest header before this word
-                if ((int)x < (int)EVENT_BEGIN)           // a road header
-                    hdr[r + 1] = make_uint2(first + 32 * i, x);
+                if ((int)x < (int)EVENT_BEGIN) {         // a road header
+                    if constexpr (PAIR) {
+                        hdr_pos[r + 1] = (uint16_t)(first + 32 * i);
+                        hdr_word[r + 1] = x;
+                    } else {
+                        hdr[r + 1] = make_uint2(first + 32 * i, x);
+                    }
+                }
                 // the first word of a run of hits of one layer (in this row)
                 if ((hit & (!same | (lane == 0))) & (r >= 0)) {
                     const uint32_t len = (uint32_t)(__clz((int)__brev(~sm & (0xFFFFFFFEu << lane))) - lane);
@@ -512,7 +522,9 @@ __global__ void __launch_bounds__(TILE_THREADS, 12)
             const uint32_t r = tile_base + rl;
             uint32_t items = 0;
             if (rl < n_roads_tile) {
-                const uint32_t p = tile_start + hdr[rl].x, hw = hdr[rl].y, packed = cnt[rl];
+                const uint32_t p = tile_start + (PAIR ? hdr_pos[PAIR ? rl : 0] : hdr[PAIR ? 0 : rl].x);
+                const uint32_t hw = PAIR ? hdr_word[PAIR ? rl : 0] : hdr[PAIR ? 0 : rl].y;
+                const uint32_t packed = cnt[rl];
                 if (rd_sector(hw) >= cfg.n_sectors) report(status, p, SVT_ERR_BAD_SECTOR);      // V9
                 if (PAIR) {
                     // V11, at the last word of the road's run.  A run of more than 96
@@ -606,18 +618,19 @@ void launch_unpack_roads(const uint32_t *words, const uint64_t *event_off, const
                          unsigned long long *tile_state, uint32_t *tile_ticket, uint64_t *total64,
                          uint64_t road_cap, uint32_t *road_word, uint32_t *road_nhit,
                          uint32_t *event_road, const svt_config cfg, const FusedRoads fr,
-                         uint64_t *counts, unsigned long long *status, int grid, bool max_shared,
-                         cudaStream_t st) {
+                         uint64_t *counts, unsigned long long *status, int grid,
+                         bool max_shared, cudaStream_t st) {
     uint64_t T = n_tiles(max_words);
     int g = (int)(T < (uint64_t)grid ? T : (uint64_t)grid);
     if (g < 1) g = 1;   // an empty batch still writes its road count
-    // max_shared: the fit kernel with one road per lane needs 171 KB of shared
-    // memory on an SM, this one alone 164, and an SM has to run empty to change
-    // its split: with the larger split from here on the fit's blocks start
-    // beside the last tiles (3000 events of small roads, whole pass: 41.6 us
-    // without, 37.0 with).  The other forms of the fit need all 228 KB; asking
-    // for it here already changed nothing (3000 events: 206.3 and 206.2) or
-    // cost 3 % (512 events of uneven roads), so it is left to their launch.
+    // max_shared (the fit kernel with one road per lane comes next and the words
+    // are in device memory): an SM has to run empty to change how its on-chip
+    // memory is split, and with this kernel's own choice (164 KB of shared memory)
+    // the fit's blocks cannot start beside the last tiles.  3000 events of small
+    // roads, whole pass: 41.6 us without, 38.2 with.  Words in mapped host memory
+    // want the L1 that the larger split takes: 97 us without, 115 with.  The
+    // other forms of the fit gained nothing (3000 events: 206.3 and 206.2) or
+    // lost 3 % (512 events of uneven roads).
     launch_chained(max_shared, cfg.xft_pairs ? k_unpack_roads<true> : k_unpack_roads<false>, g, TILE_THREADS, 0, st, words, event_off, dims, first_ev,
                  tile_state, tile_ticket, total64, road_cap, road_word, road_nhit, event_road, cfg,
                  fr, counts, status);
