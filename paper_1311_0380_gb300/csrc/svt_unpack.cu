@@ -184,9 +184,9 @@ __device__ unsigned long long tiles_before(const unsigned long long *state, uint
 // 56 roads' descriptors; 62 % of the slots taken at 12 tiles per SM) and the
 // chain of loads, barriers and look-back of a tile, not by HBM.  Before, a
 // thread took eight consecutive words and block scans and barriers (nine a tile)
-// joined them.  Alone on the GPU with warm caches, before and now: 1 tile 8.6
-// and 6.4 us, 115 tiles 10.4 and 8.6, 1222 tiles 14.2 and 12.7, 3441 tiles 29.5
-// and 24.5, 7694 tiles 47.7 and 43.6.  (Windows of 64 or 128 tiles in the
+// joined them.  Alone on the GPU, before and now: cold caches, 1 tile 8.6
+// and 6.4 us, 115 tiles 10.4 and 8.6; warm, 1222 tiles 14.2 and 12.7, 3441 29.5
+// and 24.5, 7694 47.7 and 43.6.  (Windows of 64 or 128 tiles in the
 // look-back gained nothing; the instances differ by the pairing's counts, whose
 // code costs 5 % where it is not used.)
 template <bool PAIR>
