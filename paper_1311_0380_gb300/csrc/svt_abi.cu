@@ -153,8 +153,11 @@ CalibIndex carve_calib_index(const void *base, uint64_t n, uint32_t S) {
     Carver c(const_cast<void *>(base));
     CalibIndex x;
     x.max_items = calib_max_items(n, S);
-    x.counts = c.take<uint32_t>((size_t)S * calib_tiles(n) + 1);
-    x.totals = c.take<uint32_t>(S);
+    // the sectors' totals follow their counts; the counts of a single tile are
+    // the totals (svt_calib_index_size must not grow: callers keep its value)
+    const size_t T = calib_tiles(n);
+    x.counts = c.take<uint32_t>(S * (T > 1 ? T + 1 : T) + 1);
+    x.totals = T > 1 && x.counts ? x.counts + S * T : x.counts;
     x.sector_off = c.take<int32_t>(S + 1);
     x.sector_item = c.take<int32_t>(S + 1);
     x.item_sector = c.take<int32_t>(x.max_items);

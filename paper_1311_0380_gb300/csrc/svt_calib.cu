@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
 }
 
 // block s: exclusive scan of sector s's counts over the tiles, and its total
+// (a single tile has no scan: its counts are the totals)
 __global__ void __launch_bounds__(SORT_THREADS)
     k_sector_scan(uint32_t *counts, uint32_t T, uint32_t *totals) {
     __shared__ uint32_t sm[SORT_WARPS + 1];
@@ -201,7 +202,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 2)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const uint32_t s = threadIdx.x * 2 + h;
-            first[h] = s < S ? (uint32_t)sector_off[s] + base[(uint64_t)s * T + t] : 0u;
+            first[h] = s < S ? (uint32_t)sector_off[s] + (T > 1 ? base[(uint64_t)s * T + t] : 0u) : 0u;
         }
         for (int k = threadIdx.x; k < SORT_WARPS * 512 / 2; k += SORT_THREADS)
             reinterpret_cast<uint32_t *>(cnt)[k] = 0;
@@ -1444,7 +1445,7 @@ cudaError_t launch_calib_sort(const int32_t *sector, uint64_t n, uint32_t S, uin
     }
     const int g = (int)min((uint32_t)(max(sms, 1) * 8), T);
     k_hist<<<g, SORT_THREADS, 0, st>>>(sector, n, S, T, counts, status);
-    launch_after(k_sector_scan, S, SORT_THREADS, 0, st, counts, T, totals);
+    if (T > 1) launch_after(k_sector_scan, S, SORT_THREADS, 0, st, counts, T, totals);
     launch_after(k_items, (int)min(calib_max_items(n, S) / 512 + 1, (uint32_t)max(sms, 1)), 512, 0,
                  st, (const uint32_t *)totals, S, n, sector_off, sector_item, item_sector,
                  item_start, n_items, calib_max_items(n, S));
