@@ -847,15 +847,21 @@ constexpr uint32_t NONE = 0xFFFFFFFFu;
 constexpr uint32_t LIST_MAX = 8, CAND = 96;
 struct CandList {
     uint2 ent[32];        // road, combination
-    uint2 cand[CAND];     // combinations of the road at hand that are within reach,
-                          // each with the bits of its s
 };
+static_assert(sizeof(CandList) <= sizeof(RecordList), "a warp's list holds either form");
 
-// flush_records works where the road's tables were: per entry six record words,
-// 18 words of F (19: odd, so that the lanes' reads fall in different banks),
-// three of q
+// A road's tables and the combinations of it that are within reach, each with
+// the bits of its s; flush_records works in the same place between roads: per
+// entry six record words, 18 words of F (19: odd, so that the lanes' reads fall
+// in different banks), three of q.  The candidates sit in the slot, which is
+// larger than the tables, and not beside the list: with 1024 bytes of list a
+// warp instead of 384 blocks of four warps fitted seven times on an SM and not
+// eight (of two 15 and 16, of one 28 and 30).
 union ScreenSlot {
-    ScreenSmem road;
+    struct {
+        ScreenSmem road;
+        uint2 cand[CAND];
+    };
     uint32_t flush[32 * (6 + 19 + 3)];
 };
 static_assert(sizeof(ScreenSlot) <= sizeof(WarpSmem) && alignof(ScreenSlot) <= 16,
@@ -1461,8 +1467,8 @@ __device__ __forceinline__ uint32_t screen_path(
         const uint32_t a_lo = k * fr.rows;
         const uint32_t a_hi = min(a_lo + fr.rows, g.NA);
         float thr;
-        const uint32_t n_c = list_rows(sm, rl.cand, g, a_lo, a_hi, sc, thr, (uint32_t)lane);
-        const unsigned long long best = best_of_list(sm, rl.cand, n_c, thr, a_lo * g.NB,
+        const uint32_t n_c = list_rows(sm, slot.cand, g, a_lo, a_hi, sc, thr, (uint32_t)lane);
+        const unsigned long long best = best_of_list(sm, slot.cand, n_c, thr, a_lo * g.NB,
                                                      min(a_hi * g.NB, g.C_eval), cfg, LW);
         uint32_t last = 0;
         if (lane == 0) {
@@ -1499,11 +1505,11 @@ __device__ __forceinline__ uint32_t screen_path(
             const RoadDesc D = shfl_desc(da, db, jj);
             if (D.a.w > fr.small_max) continue;   // split road: done above
             if (n_rec > 32u - LIST_MAX) flush();
-            const uint32_t n_c = screen_road(sm, rl.cand, words, D, F, q, cfg, sc, LW);
+            const uint32_t n_c = screen_road(sm, slot.cand, words, D, F, q, cfg, sc, LW);
             __syncwarp();
             const uint32_t n_e = max(n_c, 1u);   // at most LIST_MAX
             if ((uint32_t)lane < n_e)
-                rl.ent[n_rec + lane] = make_uint2(c0 + jj, n_c ? rl.cand[lane].x : NONE);
+                rl.ent[n_rec + lane] = make_uint2(c0 + jj, n_c ? slot.cand[lane].x : NONE);
             n_rec += n_e;
             __syncwarp();
         }
@@ -1512,11 +1518,6 @@ __device__ __forceinline__ uint32_t screen_path(
     return n_pass;
 }
 
-// a warp's list beside its slot (GROUP 1 screens and lists candidates as well)
-template <int GROUP>
-constexpr size_t LIST_BYTES = GROUP == 1 && sizeof(CandList) > sizeof(RecordList)
-                                  ? sizeof(CandList) : sizeof(RecordList);
-static_assert(LIST_BYTES<1> % 16 == 0 && LIST_BYTES<32> % 16 == 0, "lists keep 16-byte alignment");
 // Mean evaluated combinations of a batch's roads from which on the batch is
 // fitted by screening (one road per warp, GROUP 1; one form per launch, so that
 // the warps keep to one path of code).  Its set-up, listing and exact step cost
@@ -1554,7 +1555,7 @@ __global__ void __launch_bounds__(GROUP == 32 ? 384 : 512, 2)
                      uint32_t roads_per_chunk, uint32_t *out, unsigned long long *status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     WarpSmem &sm = *reinterpret_cast<WarpSmem *>(smem_raw + SLOT_BYTES * (threadIdx.x >> 5));
-    unsigned char *list = smem_raw + SLOT_BYTES * (blockDim.x >> 5) + LIST_BYTES<GROUP> * (threadIdx.x >> 5);
+    unsigned char *list = smem_raw + SLOT_BYTES * (blockDim.x >> 5) + sizeof(RecordList) * (threadIdx.x >> 5);
     RecordList &rl = *reinterpret_cast<RecordList *>(list);
     const int lane = threadIdx.x & 31;
     const Lanes<32> LW = lanes_of<32>(lane);
@@ -1817,8 +1818,8 @@ __global__ void __launch_bounds__(GROUP == 32 ? 384 : 512, 2)
 
 }  // namespace
 
-size_t fit_smem_bytes(int warps_per_block, uint32_t group) {
-    return (SLOT_BYTES + (group == 1 ? LIST_BYTES<1> : LIST_BYTES<32>)) * (size_t)warps_per_block;
+size_t fit_smem_bytes(int warps_per_block) {
+    return (SLOT_BYTES + sizeof(RecordList)) * (size_t)warps_per_block;
 }
 
 namespace {
@@ -1841,7 +1842,7 @@ Screen make_screen(const svt_config &cfg) {
 
 
 int fit_persistent_blocks_per_sm(int warps_per_block, uint32_t group) {
-    const size_t smem = fit_smem_bytes(warps_per_block, group);
+    const size_t smem = fit_smem_bytes(warps_per_block);
     int occ = 1 << 30;
     auto one = [&](auto kernel) {
         int n = 0;
@@ -1875,7 +1876,7 @@ cudaError_t launch_fit_persistent(const uint32_t *words, const uint64_t *event_o
                                   const FusedRoads fr, uint32_t roads_per_chunk, uint32_t group,
                                   uint32_t *out, unsigned long long *status,
                                   int warps_per_block, int grid, cudaStream_t st) {
-    const size_t smem = fit_smem_bytes(warps_per_block, group);
+    const size_t smem = fit_smem_bytes(warps_per_block);
     const bool guarded = cfg.chi2_cut < SAT;
     const Screen sc = make_screen(cfg);
     auto launch = [&](auto kernel) {

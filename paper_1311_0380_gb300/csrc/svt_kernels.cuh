@@ -127,7 +127,7 @@ cudaError_t launch_fit_persistent(const uint32_t *words, const uint64_t *event_o
 // persistent blocks of the fit kernel per SM for a block size and a road
 // grouping (1, 2, 4 or 32; both chi2-cut instances of it)
 int fit_persistent_blocks_per_sm(int warps_per_block, uint32_t group);
-size_t fit_smem_bytes(int warps_per_block, uint32_t group);
+size_t fit_smem_bytes(int warps_per_block);
 
 // ---- plain path (svt_plain.cu) --------------------------------------------------
 // Every plain-path kernel returns at once when *status already holds an error.
