@@ -812,7 +812,7 @@ __device__ __forceinline__ bool form_record(const uint32_t *__restrict__ words,
 // So below SAT = 32767^2 the clamped and the unclamped chi2 order alike, the
 // screen starts at reach(min(cut, SAT), delta), and when nothing below SAT
 // turns up while the cut would let larger values pass, every combination of
-// the road (or item) is evaluated exactly (sweep).
+// the road (or item) is evaluated exactly (see unsure).
 struct Screen {
     float f_scale, q_scale;   // 2^-oshift, 2^(qshift - oshift)
     float delta, thr;         // delta; reach(min(cut, SAT), delta)
@@ -1193,6 +1193,7 @@ __device__ __forceinline__ uint32_t list_rows(ScreenSmem &sm, uint2 *cand, const
                                                  __float_as_uint(s));
                         listed += __popc(hits);
                     }
+                    if (listed > CAND) return listed;   // (uniform)
                 }
             }
         }
@@ -1214,16 +1215,16 @@ __device__ __forceinline__ uint32_t list_rows(ScreenSmem &sm, uint2 *cand, const
     return listed;
 }
 
-// Best key of rows [a_lo, a_hi) by a whole warp: the listed combinations, or all
-// of them where they did not fit the list or nothing is sure to lie below SAT
-// (see Screen), evaluated exactly.
+// Whether the list of rows [a_lo, a_hi) does not decide: it did not hold all that
+// is within reach, or nothing is sure to lie below SAT (see Screen).
+__device__ __forceinline__ bool unsure(uint32_t listed, float thr, const svt_config &cfg) {
+    return listed > CAND || (cfg.chi2_cut >= SAT && !(thr < (float)SAT));
+}
+
+// Best key of the listed combinations, evaluated exactly by a whole warp.
 __device__ __forceinline__ unsigned long long best_of_list(const ScreenSmem &sm, const uint2 *cand,
-                                                           uint32_t listed, float thr,
-                                                           uint32_t c_lo, uint32_t c_hi,
-                                                           const svt_config &cfg,
+                                                           uint32_t listed, const svt_config &cfg,
                                                            const Lanes<32> &L) {
-    if (listed > CAND || (cfg.chi2_cut >= SAT && !(thr < (float)SAT)))
-        return sweep(sm, c_lo, c_hi, cfg, L);
     unsigned long long best = ~0ull;
     for (uint32_t k = L.gl; k < listed; k += 32u) {
         const uint32_t c = cand[k].x, chi2 = exact_chi2(sm, c, cfg);
@@ -1238,7 +1239,8 @@ __device__ __forceinline__ unsigned long long best_of_list(const ScreenSmem &sm,
 constexpr uint32_t DIRECT = 2;
 
 // One road fitted whole by the warp: its candidates in cand, their number
-// returned (at most LIST_MAX).
+// returned (at most LIST_MAX, or UNSURE).
+constexpr uint32_t UNSURE = 0xFFFFFFFFu;
 __device__ __forceinline__ uint32_t screen_road(ScreenSmem &sm, uint2 *cand,
                                               const uint32_t *__restrict__ words,
                                               const RoadDesc &D, const int16_t *__restrict__ F,
@@ -1255,8 +1257,9 @@ __device__ __forceinline__ uint32_t screen_road(ScreenSmem &sm, uint2 *cand,
         screen_suffix(sm, g, L);
         float thr;
         const uint32_t n = list_rows(sm, cand, g, 0, g.NA, sc, thr, L.gl);
-        if (n <= LIST_MAX && (cfg.chi2_cut < SAT || thr < (float)SAT)) return n;
-        best = best_of_list(sm, cand, n, thr, 0, g.C_eval, cfg, L);
+        if (unsure(n, thr, cfg)) return UNSURE;
+        if (n <= LIST_MAX) return n;
+        best = best_of_list(sm, cand, n, cfg, L);
     }
     __syncwarp();
     if (L.gl == 0) cand[0].x = (uint32_t)best;   // (UINT64_MAX reads as NONE)
@@ -1436,6 +1439,17 @@ __device__ __forceinline__ uint32_t chunk_first(uint32_t k, uint32_t n_full, uin
 // The fit of a whole batch by screening: items of split roads, then chunks of
 // consecutive roads, each road by one warp.  Returns the passing roads whose
 // records this lane wrote.
+// A road or item whose list does not decide (many equal hits, shifts that leave
+// few bits of chi2, every component saturated) is fitted by the exact form in the
+// same slot; after such an item the warp screens one in 2, 4, 8, then 16 of the
+// items that follow until one is decided.  Batches of such roads only, kernel and
+// extraction, in us, the exact form for every road / this / every combination
+// with digits of its own, which it did before: roads of 4096 combinations with
+// equal hits, 256 of them 47 / 31 / 90, 25,600 131 / 168 / 730; of 15,625
+// combinations (split) 33 / 39 / 116 and 441 / 487 / 3704; chi2 above SAT and no
+// cut, 25,600 roads 132 / 111 / 299 and 441 / 471 / 976.  (Leaving the screen out
+// for roads as well takes 168 to 149, but 1.5 % more for every other batch.)
+template <bool GUARDED>
 __device__ __forceinline__ uint32_t screen_path(
     ScreenSlot &slot, CandList &rl, const uint32_t *__restrict__ words,
     const RoadDesc *__restrict__ desc, const int16_t *__restrict__ F,
@@ -1450,6 +1464,20 @@ __device__ __forceinline__ uint32_t screen_path(
         n_pass += flush_records(words, desc, F, q, cfg, out, rl, slot.flush, n_rec);
         n_rec = 0;
     };
+    uint32_t skip = 0;   // the screen is left out where this mask hits the item's number
+    // best (chi2 << 32) | c of rows [a_lo, a_hi), every combination exactly
+    auto exact = [&](const RoadDesc &D, const Geo &g, uint32_t a_lo, uint32_t a_hi) {
+        const uint32_t sh = 32u - cfg.oshift;
+        const uint32_t init_chi = cfg.chi2_cut == 0xFFFFFFFFu ? 0xFFFFFFFFu : cfg.chi2_cut + 1u;
+        WarpSmem &ws = reinterpret_cast<WarpSmem &>(slot);
+        __syncwarp();
+        road_setup<32>(ws, words, D, g, F, q, sh, cfg.xft_pairs, kColBias<GUARDED>, LW);
+        const unsigned long long k =
+            eval_rows<GUARDED, 32>(ws, g, a_lo, a_hi, cfg.qshift + sh, init_chi, LW);
+        const uint32_t low = (uint32_t)k;
+        __syncwarp();
+        return k == ~0ull ? k : (k & 0xFFFFFFFF00000000ull) | ((low >> 9) * g.NB + (low & 511u));
+    };
     while (n_items) {   // (no items: no claim, 3.5 us of queueing for a grid's warps)
         uint32_t it = 0;
         if (lane == 0) it = atomicAdd(bl.counters + 0, 1u);
@@ -1462,14 +1490,19 @@ __device__ __forceinline__ uint32_t screen_path(
         D.a = __ldg(&desc[r].a);
         D.b = __ldg(&desc[r].b);
         const Geo g = geo_of(D);
-        screen_load(sm, words, D, g, F, q, sc, cfg.xft_pairs, LW);
-        screen_suffix(sm, g, LW);
         const uint32_t a_lo = k * fr.rows;
         const uint32_t a_hi = min(a_lo + fr.rows, g.NA);
-        float thr;
-        const uint32_t n_c = list_rows(sm, slot.cand, g, a_lo, a_hi, sc, thr, (uint32_t)lane);
-        const unsigned long long best = best_of_list(sm, slot.cand, n_c, thr, a_lo * g.NB,
-                                                     min(a_hi * g.NB, g.C_eval), cfg, LW);
+        uint32_t n_c = UNSURE;
+        if ((it & skip) == 0) {
+            screen_load(sm, words, D, g, F, q, sc, cfg.xft_pairs, LW);
+            screen_suffix(sm, g, LW);
+            float thr;
+            n_c = list_rows(sm, slot.cand, g, a_lo, a_hi, sc, thr, (uint32_t)lane);
+            if (unsure(n_c, thr, cfg)) n_c = UNSURE;
+            skip = n_c == UNSURE ? (2u * skip + 1u) & 15u : 0u;
+        }
+        const unsigned long long best = n_c == UNSURE ? exact(D, g, a_lo, a_hi)
+                                                      : best_of_list(sm, slot.cand, n_c, cfg, LW);
         uint32_t last = 0;
         if (lane == 0) {
             if (best != ~0ull) atomicMin(fr.key + r, best);
@@ -1505,7 +1538,15 @@ __device__ __forceinline__ uint32_t screen_path(
             const RoadDesc D = shfl_desc(da, db, jj);
             if (D.a.w > fr.small_max) continue;   // split road: done above
             if (n_rec > 32u - LIST_MAX) flush();
-            const uint32_t n_c = screen_road(sm, slot.cand, words, D, F, q, cfg, sc, LW);
+            uint32_t n_c = screen_road(sm, slot.cand, words, D, F, q, cfg, sc, LW);
+            if (n_c == UNSURE) {
+                // (read again: kept over the screen it spills)
+                const RoadDesc E{__ldg(&desc[c0 + jj].a), __ldg(&desc[c0 + jj].b)};
+                const Geo g = geo_of(E);
+                const unsigned long long best = exact(E, g, 0, g.NA);
+                if (lane == 0) slot.cand[0].x = (uint32_t)best;   // (UINT64_MAX reads as NONE)
+                n_c = 1;
+            }
             __syncwarp();
             const uint32_t n_e = max(n_c, 1u);   // at most LIST_MAX
             if ((uint32_t)lane < n_e)
@@ -1577,7 +1618,7 @@ __global__ void __launch_bounds__(GROUP == 32 ? 384 : 512, 2)
         if (counts[2] >= SCREEN_MEAN * R64) {
             const uint32_t n_pass = __reduce_add_sync(
                 0xffffffffu,
-                screen_path(reinterpret_cast<ScreenSlot &>(sm), *reinterpret_cast<CandList *>(list),
+                screen_path<GUARDED>(reinterpret_cast<ScreenSlot &>(sm), *reinterpret_cast<CandList *>(list),
                             words, desc, F, q, cfg, sc, fr, n_big, n_items, R, roads_per_chunk, out));
             if (lane == 0 && n_pass)
                 atomicAdd((unsigned long long *)(counts + 3), (unsigned long long)n_pass);
