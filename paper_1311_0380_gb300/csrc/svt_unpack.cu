@@ -488,6 +488,26 @@ __global__ void __launch_bounds__(TILE_THREADS, 12)
                 }
             }
         }
+        // V11 where an event starts with a hit: the run of the road before it ends
+        // there, and not with the hits (at the offset, V1 decides against the run
+        // that the counts below cover).  A run of more than 96 hits breaks another
+        // rule at one of its own words.
+        if (PAIR && v1_flag) {
+            for (uint32_t e = e_mine; e < e_hi; e += TILE_THREADS) {
+                const uint32_t ps = event_pos(e), s0 = tile_start + ps;
+                if (ps >= TILE_WORDS || !((hit_bits[ps >> 5] >> (ps & 31u)) & 1u)) continue;
+                int unpaired = 0;
+                for (uint32_t n = 1; n <= min(s0, 97u); ++n) {
+                    const uint32_t x = __ldg(words + s0 - n);
+                    if (x >= HIT_END) {
+                        if (unpaired && (int)x < (int)EVENT_BEGIN)   // the run's road header
+                            report(status, (uint64_t)s0 - 1, SVT_ERR_XFT_UNPAIRED);
+                        break;
+                    }
+                    unpaired += (hit_layer(x) == 4 ? 1 : 0) - (hit_layer(x) == 5 ? 1 : 0);
+                }
+            }
+        }
         // V8: a hit whose 16 predecessors are hits of its layer is the 17th (or
         // later) of a run, i.e. 16 consecutive "same" bits end at it.  Lane
         // k - 1 looks at rows k - 2 and k - 1 (mask words k - 1 and k): bit i of
