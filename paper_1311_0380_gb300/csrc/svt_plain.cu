@@ -543,58 +543,70 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long ke
     return ((unsigned long long)hi << 32) | lo;
 }
 
-// Chi-square cut and best combination of each road.  A block takes
-// SELECT_GROUP consecutive roads at a time: its warps share those of at most
-// SELECT_BIG combinations, then the whole block scans each longer one.
-// Bound at the end by the longest road's block, hence the sixteen loads: with
-// eight the scaled workload's 200 events (12,800 roads, one of 100 thousand
-// combinations) take 33 us instead of 22; blocks of 512 or 1024 threads take 26
-// to 34, groups of 8 to 64 roads 22 to 32.  (Groups of 256 roads, and long roads
-// in a launch of their own, left most of the GPU waiting for a few blocks: 86 us.)
+// Chi-square cut and best combination of each road.  A block takes a group of
+// consecutive roads at a time: its warps share those of at most SELECT_BIG
+// combinations, then the whole block scans each longer one.  Bound at the end by
+// the longest road's block, hence the sixteen loads: with eight the scaled
+// workload's 200 events (12,800 roads, one of 100 thousand combinations) take
+// 33 us instead of 22; blocks of 512 or 1024 threads take 26 to 34, groups of 8 to
+// 64 roads 22 to 32.  Where the roads are short on the mean nothing is left to
+// wait for, and what counts is the latency of a group: there a group holds as many
+// roads as give every block one (at most SELECT_GROUP_MAX).  Roads of at most 64
+// combinations take two loads a lane.  In us, one warp per road over the whole
+// grid / groups of 16 from a counter in the block / now: 200,000 roads of one
+// combination 49 / 89 / 21, 96,000 of 64 27 / 44 / 14, 128,000 of 729 95 / 86 / 67,
+// the scaled workload 49 / 16.4 / 14.9 (without the rest of the stages).
 constexpr uint32_t SELECT_THREADS = 256, SELECT_GROUP = 16, SELECT_BIG = 1024;
+constexpr uint32_t SELECT_GROUP_MAX = 128, SELECT_SMALL_MEAN = 128;
 __global__ void __launch_bounds__(SELECT_THREADS)
     k_select(const uint32_t *__restrict__ fit_chi2, const int32_t *__restrict__ fit_par,
              uint64_t comb_cap, const uint64_t *__restrict__ comb_off,
              const uint32_t *__restrict__ road_flags, const uint64_t *__restrict__ n_roads,
              uint64_t road_cap, const svt_config cfg, svt_best *best,
              const unsigned long long *status) {
-    __shared__ RoadMeta meta[SELECT_GROUP];
-    __shared__ unsigned long long key_s[SELECT_GROUP];
-    __shared__ uint32_t next;
+    __shared__ RoadMeta meta[SELECT_GROUP_MAX];
+    __shared__ unsigned long long key_s[SELECT_GROUP_MAX];
     wait_prior_grid();
     allow_next_grid();
     if (!status_ok(status)) return;
     const uint64_t R = road_count(n_roads, road_cap);
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t init_chi = cfg.chi2_cut == 0xFFFFFFFFu ? 0xFFFFFFFFu : cfg.chi2_cut + 1u;
-    for (uint64_t g = (uint64_t)blockIdx.x * SELECT_GROUP; g < R;
-         g += (uint64_t)gridDim.x * SELECT_GROUP) {
-        const uint32_t n = (uint32_t)min((uint64_t)SELECT_GROUP, R - g);
-        if (threadIdx.x == 0) next = 0;
-        if (threadIdx.x < SELECT_GROUP) {
-            RoadMeta m{0, 0, 0};
-            if (threadIdx.x < n) {
-                m.off = __ldg(comb_off + g + threadIdx.x);
-                m.n = __ldg(comb_off + g + threadIdx.x + 1) - m.off;
-                m.word = __ldg(road_flags + g + threadIdx.x);
-                if (m.off + m.n > comb_cap) m.n = 0;   // (an error status by now)
-            }
+    uint32_t group = SELECT_GROUP;
+    if (R && __ldg(comb_off + R) < R * SELECT_SMALL_MEAN)
+        group = (uint32_t)max((uint64_t)SELECT_GROUP,
+                              min((R + gridDim.x - 1) / gridDim.x, (uint64_t)SELECT_GROUP_MAX));
+    for (uint64_t g = (uint64_t)blockIdx.x * group; g < R; g += (uint64_t)gridDim.x * group) {
+        const uint32_t n = (uint32_t)min((uint64_t)group, R - g);
+        bool big = false;
+        if (threadIdx.x < n) {
+            RoadMeta m;
+            m.off = __ldg(comb_off + g + threadIdx.x);
+            m.n = __ldg(comb_off + g + threadIdx.x + 1) - m.off;
+            m.word = __ldg(road_flags + g + threadIdx.x);
+            if (m.off + m.n > comb_cap) m.n = 0;   // (an error status by now)
+            big = m.n > SELECT_BIG;
             meta[threadIdx.x] = m;
             key_s[threadIdx.x] = ~0ull;
         }
-        __syncthreads();
-        for (;;) {
-            uint32_t k = 0;
-            if (lane == 0) k = atomicAdd(&next, 1u);
-            k = __shfl_sync(0xffffffffu, k, 0);
-            if (k >= n) break;
+        big = __syncthreads_or(big);
+        for (uint32_t k = threadIdx.x >> 5; k < n; k += SELECT_THREADS / 32) {
             const RoadMeta m = meta[k];
             if (m.n == 0 || m.n > SELECT_BIG) continue;
-            const unsigned long long key =
-                warp_min_key(scan_chi2<32>(fit_chi2 + m.off, m.n, init_chi, lane));
+            unsigned long long key;
+            if (m.n <= 64) {
+                const uint32_t *chi2 = fit_chi2 + m.off;
+                const uint32_t v0 = lane < m.n ? __ldg(chi2 + lane) : 0xFFFFFFFFu;
+                const uint32_t v1 = lane + 32 < m.n ? __ldg(chi2 + lane + 32) : 0xFFFFFFFFu;
+                const uint32_t v = min(v0, v1), c = v0 <= v1 ? lane : lane + 32;
+                key = v < init_chi ? ((unsigned long long)v << 32) | c : ~0ull;
+            } else {
+                key = scan_chi2<32>(fit_chi2 + m.off, m.n, init_chi, lane);
+            }
+            key = warp_min_key(key);
             if (lane == 0) key_s[k] = key;
         }
-        for (uint32_t k = 0; k < n; ++k) {
+        for (uint32_t k = 0; big && k < n; ++k) {
             const RoadMeta m = meta[k];
             if (m.n <= SELECT_BIG) continue;   // uniform over the block
             const unsigned long long key = warp_min_key(
