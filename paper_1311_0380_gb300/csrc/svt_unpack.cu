@@ -651,9 +651,9 @@ void launch_unpack_roads(const uint32_t *words, const uint64_t *event_off, const
     // want the L1 that the larger split takes: 97 us without, 115 with.  The
     // other forms of the fit gained nothing (3000 events: 206.3 and 206.2) or
     // lost 3 % (512 events of uneven roads).
-    launch_chained(max_shared, cfg.xft_pairs ? k_unpack_roads<true> : k_unpack_roads<false>, g, TILE_THREADS, 0, st, words, event_off, dims, first_ev,
-                 tile_state, tile_ticket, total64, road_cap, road_word, road_nhit, event_road, cfg,
-                 fr, counts, status);
+    launch_chained(max_shared, cfg.xft_pairs ? k_unpack_roads<true> : k_unpack_roads<false>, g,
+                   TILE_THREADS, 0, st, words, event_off, dims, first_ev, tile_state, tile_ticket,
+                   total64, road_cap, road_word, road_nhit, event_road, cfg, fr, counts, status);
 }
 
 void launch_unpack_events(const uint32_t *words, const uint64_t *event_off, const Dims *dims,
