@@ -22,11 +22,17 @@ def _p(t):
     return None if t is None else t.data_ptr()
 
 
+# not part of torch's documented interface, so a torch without it has to do
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
     # the handle alone: torch.cuda.current_stream() builds a Stream object for
     # it, 2.8 us of a call's 16 before it was left out (0.3 now)
     if stream is None:
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        if _raw_stream is None:
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(torch.cuda.current_device())
     return stream.cuda_stream
 
 
