@@ -671,7 +671,13 @@ int svt_calib_grad_scale(const float *d_scale, const float *d_dF, const float *d
                          uint32_t n_sectors, float *d_out_dF, float *d_out_dq, void *stream);
 
 /* Backward of y = F[s] x + q[s] from d_grad_y [N][6]: d_dF[s] = sum_t g_t x_t^T,
- * d_dq[s] = sum_t g_t and, when d_dx is not NULL, d_dx_t = F[s]^T g_t. */
+ * d_dq[s] = sum_t g_t and, when d_dx is not NULL, d_dx_t = F[s]^T g_t.  When d_x
+ * and d_grad_y start on 16-byte boundaries and d_dx is NULL, the tracks are staged
+ * in shared memory by bulk copies as in svt_calib_loss_grad, and the sums run over
+ * the runs of a device's warps; otherwise every lane loads its own tracks and the
+ * sums run item by item.  Each order is fixed, so repeated calls give identical
+ * bits, but the two orders round differently.  A staged copy that does not land
+ * within the pass's bounded wait makes the sums it belongs to NaN. */
 int svt_calib_backward(const float *d_x, const float *d_grad_y, uint64_t n_tracks,
                        uint32_t n_sectors, const void *d_index, const float *d_F, float *d_dF,
                        float *d_dq, float *d_dx, void *d_workspace, size_t workspace_bytes,

@@ -36,8 +36,8 @@ __device__ __forceinline__ float warp_sum(float v) {
 // Four passes: histograms of tiles of SORT_TILE tracks, a scan of every
 // sector's counts over the tiles (a block per sector), the sector offsets and
 // the item table, and the scatter.  The scans of all sectors in one block had
-// been 954 of the 1112 us of putting 4 M tracks in order; now the sort is
-// bound by moving the tracks (see k_scatter).
+// been 954 of the 1112 us of putting 4 M tracks in order; now 80 to 93 of the
+// kernels' 100 to 112 us are the scatter (see there).
 constexpr int SORT_THREADS = 256, SORT_WARPS = SORT_THREADS / 32;
 constexpr int SORT_ROUNDS = SORT_TILE / SORT_THREADS;   // tracks per thread
 
@@ -165,9 +165,11 @@ __device__ __forceinline__ void stage_floats(float *dst, const float *__restrict
 // and theta rows are staged in shared memory by asynchronous copies while the
 // ranks are formed, and written in sector order, the rows of one sector (four
 // on average with 512 sectors) as one run: each array is read and written once
-// and no other pass over the tracks is needed.  Bound by the memory system:
-// 84 bytes a track at least; 4 M tracks take 88 us (3.8 TB/s), where the rank
-// pass and the two gathers took 41 + 80 us.
+// and no other pass over the tracks is needed.  Bound by waiting on shared memory
+// (ranks, tables and rows; 16 warps per SM, short-scoreboard stalls of 8 an issue,
+// DRAM at 37 % of its peak): 4 M tracks of 84 bytes take 80 to 93 us on different
+// boxes, where the bytes alone take 49 and the rank pass and the two gathers took
+// 41 + 80.
 template <bool XT>
 __global__ void __launch_bounds__(SORT_THREADS, 2)
     k_scatter(const int32_t *__restrict__ sector, uint64_t n, uint32_t S, uint32_t T,
@@ -1109,9 +1111,12 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
 // partial for every run instead of every item.  16 M tracks in 512 sectors, this
 // kernel and the final sums: 118 us, k_grad_items and k_grad_final 155; 1 M
 // tracks 17.7 and 19.0, 30 K 9.4 and 9.7 (16 sectors: 22.3 and 34.7, 9.5 and
-// 10.2); error of dF against exact sums, relative to its norm, 1.7e-7 (16 M)
-// and 1.0e-7 (1 M), 2.4e-7 and 1.3e-7 before.  A copy that does not land within
-// the bound makes its segment's sums NaN.
+// 10.2).  With everything in L2 and calls back to back the shorter sets of many
+// sectors gain nothing: 1 M tracks in 512 sectors 14.4 and 12.5, 300 K 8.4 and
+// 8.4, from 1.5 M on 16.5 and 16.6 or faster.  Error of dF against exact sums,
+// relative to its norm, 1.65e-7 (16 M) and 1.0e-7 (1 M), 2.35e-7 and 1.3e-7
+// before.  A copy that does not land within the bound makes its segment's sums
+// NaN.
 constexpr uint32_t GB_ROWS = ST_TRACKS * 24u, GB_BUF = 2u * GB_ROWS;
 constexpr int GB_WARPS = 6;
 static_assert(32 * (NPAR + 1) * 4 <= (int)GB_ROWS && GB_ROWS % 16 == 0, "buffer");
